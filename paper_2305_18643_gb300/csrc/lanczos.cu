@@ -197,15 +197,36 @@ void launch_axpby(int dty, void* y, int dta, const void* a, const double* ca, in
 }
 
 // ---- tridiagonal eigensolver (one block): tridiag.cuh --------------------------------------
+// The recurrences walk the entries one level after the other, so they run on copies in shared
+// memory; matrices too long for it (beyond ~6,000 levels) stay in global memory.
 __global__ void __launch_bounds__(kVT) k_tridiag_lowest(const double* __restrict__ a, const double* __restrict__ b, int n,
-                                                        double* __restrict__ out_eval, double* __restrict__ vec) {
-  tridiag_lowest_block(a, b, n, out_eval, vec);
+                                                        double* __restrict__ out_eval, double* __restrict__ vec,
+                                                        int staged) {
+  extern __shared__ __align__(16) double td_smem[];
+  if (!staged) {
+    tridiag_lowest_block(a, b, n, out_eval, vec);
+    return;
+  }
+  double* sa = td_smem;
+  double* sb = sa + n;
+  double* sv = sb + n + 1;
+  for (int i = threadIdx.x; i <= n; i += blockDim.x) {
+    if (i < n) sa[i] = a[i];
+    sb[i] = b[i];
+  }
+  __syncthreads();
+  tridiag_lowest_block(sa, sb, n, out_eval, sv);
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) vec[i] = sv[i];
 }
 
 void launch_tridiag_lowest(const double* alpha, const double* beta, int n, double* out_eval, double* out_vec,
                            cudaStream_t s) {
+  const size_t smem = (4 * (size_t)n + 1) * sizeof(double);
+  const bool staged = smem <= 190 * 1024;
+  if (staged && smem > 40 * 1024) allow_max_dynamic_smem(k_tridiag_lowest);
   ProfScope ps_(K_TRIDIAG, s, 0.0);
-  k_tridiag_lowest<<<1, kVT, 0, s>>>(alpha, beta, n, out_eval, out_vec);
+  k_tridiag_lowest<<<1, kVT, staged ? smem : 0, s>>>(alpha, beta, n, out_eval, out_vec, staged ? 1 : 0);
   ED_CHECK_LAUNCH();
 }
 
