@@ -453,7 +453,9 @@ __device__ int block_lanczos(const BTable& tu, const BTable& td, uint32_t umask,
     __syncthreads();
     T* X = V0;
     T* P = V1;
-    const int nmax = pass == 0 ? kBMaxIter : m - 1;
+    // (a one-state sector has one level: the rounding left in b_1 is no second direction)
+    const int nlev = n == 1 ? 1 : kBMaxIter;
+    const int nmax = pass == 0 ? nlev : m - 1;
     for (int k = 0; k < nmax; ++k) {
       double sxw, sww, sxx;
       block_hx<T>(tu, td, sval, sU, umask, (T)u0, uni, X, P, (T)g.beta[k], mode, sxw, sww, sxx, g.bs);
@@ -478,7 +480,7 @@ __device__ int block_lanczos(const BTable& tu, const BTable& td, uint32_t umask,
       T* t = X;
       X = P;
       P = t;
-      if (pass == 0 && (stop_here || (k + 1) % kBCheck == 0 || k + 1 == kBMaxIter)) {
+      if (pass == 0 && (stop_here || (k + 1) % kBCheck == 0 || k + 1 == nlev)) {
         const int levels = k + 1;
         tridiag_lowest_block(g.alpha, g.beta, levels, g.eval, g.svec);
         __syncthreads();

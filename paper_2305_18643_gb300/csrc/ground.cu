@@ -413,7 +413,8 @@ GroundResult run_ground_state(ed_cluster& c, int dtype, double tol, int max_iter
     // normalize the start vector
     launch_dot(dt, Vs.p, dt, Vs.p, du, dd, ld, part.p, nblk + 8, scal.p + 0, s);
     axpby_inv_sqrt(dt, Vs.p, scal.p + 0, du, dd, ld, s);  // Vs <- Vs / sqrt(<Vs,Vs>)
-    LanczosRun L(std::max(2, max_iter), nblk);
+    // a one-state sector has one level: the rounding left in b_1 is no second direction
+    LanczosRun L(dim == 1 ? 1 : std::max(2, max_iter), nblk);
     const double tol_ritz = dt == ED_FP64 ? std::min(1e-2, 0.1 * tol) : 1e-7;
     bool breakdown = false;
     // the retrace accumulates the ground state in the vectors' precision (FP32 form: FP32 sum of
