@@ -1,12 +1,13 @@
 // Lattice steps that consume the cluster Green function: cluster perturbation theory (Sec. 3,
 // Eqs. CPT1-CPT3) and the CDMFT bath fit (Sec. 6, Eqs. hybridization, CPT_CDMFT, dist_func).
 //
-// All of it is small dense complex linear algebra repeated over many (k~, z) pairs, so the unit
-// of work is one warp per L x L matrix (L <= 32 cluster sites, lane = column): the matrix and its
-// inverse live in the warp's slice of shared memory and are reduced by Gauss-Jordan elimination
-// with partial pivoting (pivot row found by a warp arg-max).  Sums over k~ (the super-lattice
-// average) and over frequencies (the distance and its gradient) run in a fixed order, so repeated
-// calls give bitwise identical results.
+// All of it is small dense complex linear algebra repeated over many (k~, z) pairs, bound by the
+// FP64 pipe (two lanes per clock and SM): the unit of work is a group of M lanes per L x L matrix
+// (M = L rounded up to a power of two, 32 / M matrices per warp, lane = column), so that no lane of
+// the FP64 instructions is idle; every lane keeps its column in registers, where in-place
+// Gauss-Jordan elimination with partial pivoting turns it into a column of the inverse.  Sums over
+// k~ (the super-lattice average) and over frequencies (the distance and its gradient) run in a fixed
+// order, so repeated calls give bitwise identical results.
 //
 //   V(k~)_{ij}   = sum_bonds t e^{i k~.r~} at (i, j), its conjugate at (j, i)   (Sec. 2.2)
 //   G(k~, z)     = [G_c(z)^-1 + Gamma(z) - V(k~)]^-1                             (Eqs. CPT1, CPT_CDMFT)
@@ -17,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "ed_common.cuh"
@@ -24,7 +26,7 @@
 namespace ed {
 
 constexpr int kLatMaxSites = 32;
-constexpr int kLatWarps = 4;  // matrices per block of the inversion kernels
+constexpr int kLatThreads = 128;  // threads per block of the inversion kernels
 
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
@@ -38,78 +40,100 @@ __device__ __forceinline__ double2 cinv(double2 a) {
   return make_double2(a.x * s, -a.y * s);
 }
 
-// Inverts the L x L complex matrix a (row-major, leading dimension L) in shared memory into b,
-// one warp, lane j owning column j; col is L elements of scratch.  a is destroyed.  Returns false
-// (b undefined) if a pivot is exactly zero.
-__device__ bool warp_invert(double2* a, double2* b, double2* col, int L) {
-  const int lane = threadIdx.x & 31;
-  for (int i = 0; i < L; ++i)
-    if (lane < L) b[i * L + lane] = make_double2(i == lane ? 1.0 : 0.0, 0.0);
-  __syncwarp();
+__device__ __forceinline__ double2 shfl2(double2 v, int src, int width) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src, width), __shfl_sync(0xffffffffu, v.y, src, width));
+}
+
+// In-place inverse of an L x L complex matrix by a group of M lanes (a power of two >= L), lane j
+// holding column j in c[0, L).  Gauss-Jordan elimination; the pivot of step k is the remaining row
+// whose entry in column k has the largest max(|re|, |im|) (within sqrt(2) of the largest modulus;
+// compared as integers, off the FP64 pipe).  The rows rotate through the registers, so that the
+// pivot row is always c[0] and every register index is static.  On return lane j holds column `dst`
+// of the inverse (row swaps become column swaps).  Returns false if a pivot is zero or NaN.  All
+// lanes of the warp must call it.
+template <int M>
+__device__ __forceinline__ bool group_invert(double2 (&c)[M], int L, int& dst) {
+  const int j = threadIdx.x & (M - 1);
   bool ok = true;
+  int prow = j;  // pivot row of step k, kept by lane k
   for (int k = 0; k < L; ++k) {
-    // pivot: the row i >= k with the largest |a[i][k]| (smallest i on ties)
-    double best = lane >= k && lane < L ? cabs2(a[lane * L + k]) : -1.0;
-    int bi = lane;
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
+    int p = 0;
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      if (i < L - k) {
+        const unsigned long long r = (unsigned long long)__double_as_longlong(c[i].x) << 1;
+        const unsigned long long m = (unsigned long long)__double_as_longlong(c[i].y) << 1;
+        const unsigned long long v = r > m ? r : m;  // magnitudes order as their bits
+        if (i == 0 || v > best) {
+          best = v;
+          p = i;
+        }
       }
     }
-    if (!(best > 0.0)) ok = false;
-    if (bi != k && lane < L) {
-      double2 t = a[k * L + lane];
-      a[k * L + lane] = a[bi * L + lane];
-      a[bi * L + lane] = t;
-      t = b[k * L + lane];
-      b[k * L + lane] = b[bi * L + lane];
-      b[bi * L + lane] = t;
+    p = __shfl_sync(0xffffffffu, p, k, M);
+    best = __shfl_sync(0xffffffffu, best, k, M);
+    if (best == 0ull || best > (0x7ff0000000000000ull << 1)) ok = false;
+    if (j == k) prow = k + p;
+    // swaps by selects on values (a branch on i == p would index the registers)
+    const double2 top = c[0];
+    double2 r = top;
+#pragma unroll
+    for (int i = 1; i < M; ++i) {
+      const double2 v = c[i];
+      const bool h = i < L && i == p;
+      r = make_double2(h ? v.x : r.x, h ? v.y : r.y);
+      c[i] = make_double2(h ? top.x : v.x, h ? top.y : v.y);
     }
-    __syncwarp();
-    const double2 inv = ok ? cinv(a[k * L + k]) : make_double2(0.0, 0.0);
-    __syncwarp();
-    if (lane < L) {
-      a[k * L + lane] = cmul(a[k * L + lane], inv);
-      b[k * L + lane] = cmul(b[k * L + lane], inv);
-      col[lane] = a[lane * L + k];
-    }
-    __syncwarp();
-    if (lane < L) {
-      const double2 ak = a[k * L + lane], bk = b[k * L + lane];
-      for (int i = 0; i < L; ++i) {
-        if (i == k) continue;
-        const double2 f = col[i];
-        a[i * L + lane] = csub(a[i * L + lane], cmul(f, ak));
-        b[i * L + lane] = csub(b[i * L + lane], cmul(f, bk));
+    const double2 inv = cinv(shfl2(r, k, M));
+    const double2 f0 = j == k ? inv : cmul(r, inv);  // the scaled pivot row
+#pragma unroll
+    for (int i = 1; i < M; ++i) {
+      if (i < L) {
+        const double2 f = shfl2(c[i], k, M);
+        const double2 b = j == k ? make_double2(0.0, 0.0) : c[i];
+        c[i - 1] = make_double2(fma(f.y, f0.y, fma(-f.x, f0.x, b.x)), fma(-f.y, f0.x, fma(-f.x, f0.y, b.y)));
       }
     }
-    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      const double2 v = c[i];
+      const bool h = i == L - 1;
+      c[i] = make_double2(h ? f0.x : v.x, h ? f0.y : v.y);
+    }
+  }
+  dst = j;
+  for (int k = L - 1; k >= 0; --k) {
+    const int pk = __shfl_sync(0xffffffffu, prow, k, M);
+    dst = dst == k ? pk : dst == pk ? k : dst;
   }
   return ok;
 }
 
-// Shared memory of one warp: matrix, inverse, pivot column.
-__host__ __device__ inline size_t warp_slice(int L) { return (size_t)(2 * L * L + 32) * sizeof(double2); }
-
 // out[m] = (in[m] (+ add[m]))^-1 for count matrices; status[0] counts singular ones.
-__global__ void k_invert(const double2* __restrict__ in, const double2* __restrict__ add, double2* __restrict__ out, int L,
-                         int64_t count, int* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char lat_smem[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double2* a = reinterpret_cast<double2*>(lat_smem + w * warp_slice(L));
-  double2* b = a + L * L;
-  double2* col = b + L * L;
-  for (int64_t m = (int64_t)blockIdx.x * kLatWarps + w; m < count; m += (int64_t)gridDim.x * kLatWarps) {
-    const double2* src = in + m * L * L;
-    for (int e = lane; e < L * L; e += 32) a[e] = add ? cadd(src[e], add[m * L * L + e]) : src[e];
-    __syncwarp();
-    const bool ok = warp_invert(a, b, col, L);
-    for (int e = lane; e < L * L; e += 32) out[m * L * L + e] = b[e];
-    if (!ok && lane == 0) atomicAdd(status, 1);
-    __syncwarp();
+template <int M>
+__global__ void __launch_bounds__(kLatThreads) k_invert(const double2* __restrict__ in, const double2* __restrict__ add,
+                                                        double2* __restrict__ out, int L, int64_t count,
+                                                        int* __restrict__ status) {
+  const int j = threadIdx.x & (M - 1), g = threadIdx.x / M;
+  constexpr int G = kLatThreads / M;
+  for (int64_t m0 = (int64_t)blockIdx.x * G; m0 < count; m0 += (int64_t)gridDim.x * G) {
+    const int64_t m = m0 + g < count ? m0 + g : count - 1;  // groups past the end repeat the last matrix
+    const int jj = j < L ? j : 0;
+    double2 c[M] = {};
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      if (i < L) {
+        c[i] = in[(m * L + i) * L + jj];
+        if (add) c[i] = cadd(c[i], add[(m * L + i) * L + jj]);
+      }
+    int dst;
+    const bool ok = group_invert<M>(c, L, dst);
+    if (m0 + g >= count) continue;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      if (i < L && j < L) out[(m * L + i) * L + dst] = c[i];
+    if (!ok && j == 0) atomicAdd(status, 1);
   }
 }
 
@@ -135,91 +159,150 @@ __global__ void k_build_v(const double* __restrict__ kt, int nk, int D, const in
   }
 }
 
-// CPT: warp per (k, z) pair.  mode 0 writes G(k, z); mode 1 the periodized scalar (Eq. CPT3).
-__global__ void k_cpt(const double2* __restrict__ Gci, const double2* __restrict__ V, const double* __restrict__ kt,
-                      const double* __restrict__ pos, int D, int L, int nz, int nk, int mode, double2* __restrict__ out,
-                      int* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char lat_smem[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double2* a = reinterpret_cast<double2*>(lat_smem + w * warp_slice(L));
-  double2* b = a + L * L;
-  double2* col = b + L * L;
-  const int64_t pairs = (int64_t)nk * nz;
-  for (int64_t pr = (int64_t)blockIdx.x * kLatWarps + w; pr < pairs; pr += (int64_t)gridDim.x * kLatWarps) {
-    const int k = (int)(pr / nz), n = (int)(pr % nz);
-    for (int e = lane; e < L * L; e += 32) a[e] = csub(Gci[(int64_t)n * L * L + e], V[(int64_t)k * L * L + e]);
-    __syncwarp();
-    const bool ok = warp_invert(a, b, col, L);
-    if (!ok && lane == 0) atomicAdd(status, 1);
-    if (mode == 0) {
-      for (int e = lane; e < L * L; e += 32) out[pr * L * L + e] = b[e];
-    } else {
-      // (1/L) sum_{R R'} e^{-i k.(R - R')} G_{R R'}: lane R' sums its column, then the warp adds
-      double2 s = make_double2(0.0, 0.0);
-      if (lane < L) {
-        for (int r = 0; r < L; ++r) {
-          double ph = 0.0;
-          for (int d = 0; d < D; ++d) ph += kt[k * D + d] * (pos[r * D + d] - pos[lane * D + d]);
-          double sn, cs;
-          sincos(-ph, &sn, &cs);
-          s = cadd(s, cmul(make_double2(cs, sn), b[r * L + lane]));
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        s.x += __shfl_down_sync(0xffffffffu, s.x, o);
-        s.y += __shfl_down_sync(0xffffffffu, s.y, o);
-      }
-      if (lane == 0) out[pr] = make_double2(s.x / L, s.y / L);
-    }
-    __syncwarp();
+// ph[k][R] = e^{-i k.r_R}, the phases of the periodization (Eq. CPT3).
+__global__ void k_site_phases(const double* __restrict__ kt, const double* __restrict__ pos, int D, int L, int nk,
+                              double2* __restrict__ ph) {
+  const int64_t n = (int64_t)nk * L;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    const int k = (int)(t / L), r = (int)(t % L);
+    double x = 0.0;
+    for (int d = 0; d < D; ++d) x += kt[k * D + d] * pos[r * D + d];
+    double sn, cs;
+    sincos(-x, &sn, &cs);
+    ph[t] = make_double2(cs, sn);
   }
 }
 
-// Super-lattice average: block per frequency; warp w inverts k = w, w + kLatWarps, ... and keeps
-// its running sum in shared memory; the warps' sums are added in warp order.
-__global__ void k_cpt_average(const double2* __restrict__ Gci, const double2* __restrict__ V, int L, int nz, int nk,
-                              double2* __restrict__ out, int* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char lat_smem[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double2* a = reinterpret_cast<double2*>(lat_smem + w * warp_slice(L));
-  double2* b = a + L * L;
-  double2* col = b + L * L;
-  double2* acc = reinterpret_cast<double2*>(lat_smem + kLatWarps * warp_slice(L)) + w * L * L;
-  for (int n = blockIdx.x; n < nz; n += gridDim.x) {
-    for (int e = lane; e < L * L; e += 32) acc[e] = make_double2(0.0, 0.0);
-    for (int k = w; k < nk; k += kLatWarps) {
-      for (int e = lane; e < L * L; e += 32) a[e] = csub(Gci[(int64_t)n * L * L + e], V[(int64_t)k * L * L + e]);
-      __syncwarp();
-      const bool ok = warp_invert(a, b, col, L);
-      if (!ok && lane == 0) atomicAdd(status, 1);
-      for (int e = lane; e < L * L; e += 32) acc[e] = cadd(acc[e], b[e]);
-      __syncwarp();
+// CPT: a group of M lanes per (k, z) pair.  mode 0 writes G(k, z); mode 1 the periodized scalar
+// (Eq. CPT3).  FP64-bound: 4 L^3 multiply-adds per pair for the inverse.  On 4096 k x 256 z of 2x2
+// clusters one warp per matrix in shared memory (4 of 32 lanes busy, a sincos per matrix element)
+// took 26.4 ms, this form 1.16 ms.
+template <int M>
+__global__ void __launch_bounds__(kLatThreads) k_cpt(const double2* __restrict__ Gci, const double2* __restrict__ V,
+                                                     const double2* __restrict__ ph, int L, int nz, int nk, int mode,
+                                                     double2* __restrict__ out, int* __restrict__ status) {
+  const int j = threadIdx.x & (M - 1), g = threadIdx.x / M;
+  constexpr int G = kLatThreads / M;
+  const int64_t pairs = (int64_t)nk * nz;
+  const int jj = j < L ? j : 0;
+  for (int64_t p0 = (int64_t)blockIdx.x * G; p0 < pairs; p0 += (int64_t)gridDim.x * G) {
+    const int64_t pr = p0 + g < pairs ? p0 + g : pairs - 1;  // groups past the end repeat the last pair
+    const int64_t k = pr / nz, n = pr - k * nz;
+    double2 c[M] = {};
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      if (i < L) c[i] = csub(Gci[(n * L + i) * L + jj], V[(k * L + i) * L + jj]);
+    int dst;
+    const bool ok = group_invert<M>(c, L, dst);
+    const bool mine = p0 + g < pairs;
+    if (!ok && j == 0 && mine) atomicAdd(status, 1);
+    if (mode == 0) {
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+        if (i < L && j < L && mine) out[(pr * L + i) * L + dst] = c[i];
+    } else {
+      // (1/L) sum_{R R'} e^{-i k.(R - R')} G_{R R'}: lane R' sums its column, then the group adds
+      double2 s = make_double2(0.0, 0.0);
+      if (j < L) {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+          if (i < L) s = cadd(s, cmul(ph[k * L + i], c[i]));
+        s = cmul(s, cconj(ph[k * L + dst]));
+      }
+      for (int o = M / 2; o > 0; o >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o, M);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o, M);
+      }
+      if (j == 0 && mine) out[pr] = make_double2(s.x / L, s.y / L);
     }
+  }
+}
+
+// Super-lattice average: block per frequency; group g inverts k = g, g + G, ... and keeps its
+// running sum in registers; the groups' sums are added in group order.
+template <int M>
+__global__ void __launch_bounds__(kLatThreads) k_cpt_average(const double2* __restrict__ Gci, const double2* __restrict__ V,
+                                                             int L, int nz, int nk, double2* __restrict__ out,
+                                                             int* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char lat_smem[];
+  double2* acc0 = reinterpret_cast<double2*>(lat_smem);  // [G][L][L]
+  const int j = threadIdx.x & (M - 1), g = threadIdx.x / M;
+  constexpr int G = kLatThreads / M;
+  const int jj = j < L ? j : 0;
+  for (int n = blockIdx.x; n < nz; n += gridDim.x) {
+    double2 acc[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) acc[i] = make_double2(0.0, 0.0);
+    for (int k0 = 0; k0 < nk; k0 += G) {
+      const bool mine = k0 + g < nk;
+      const int64_t k = mine ? k0 + g : nk - 1;
+      double2 c[M] = {};
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+        if (i < L) c[i] = csub(Gci[((int64_t)n * L + i) * L + jj], V[(k * L + i) * L + jj]);
+      int dst;
+      const bool ok = group_invert<M>(c, L, dst);
+      if (!ok && j == 0 && mine) atomicAdd(status, 1);
+      // column j of the inverse is held by the lane whose dst is j
+      int src = 0;
+      for (int q = 0; q < L; ++q)
+        if (__shfl_sync(0xffffffffu, dst, q, M) == j) src = q;
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+        if (i < L) {
+          const double2 v = shfl2(c[i], src, M);
+          if (mine) acc[i] = cadd(acc[i], v);
+        }
+    }
+    __syncthreads();  // the block's previous frequency has been read
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      if (i < L && j < L) acc0[(g * L + i) * L + j] = acc[i];
     __syncthreads();
-    double2* acc0 = reinterpret_cast<double2*>(lat_smem + kLatWarps * warp_slice(L));
     for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
       double2 s = acc0[e];
-      for (int q = 1; q < kLatWarps; ++q) s = cadd(s, acc0[q * L * L + e]);
+      for (int q = 1; q < G; ++q) s = cadd(s, acc0[q * L * L + e]);
       out[(int64_t)n * L * L + e] = make_double2(s.x / nk, s.y / nk);
     }
-    __syncthreads();
   }
 }
 
-// Gamma[c][n][mu][nu] = sum_a theta[c][mu][a] theta[c][nu][a] / (z_n - eps[c][a]) (Eq. hybridization).
-__global__ void k_hybridization(const double* __restrict__ eps, const double* __restrict__ theta, const double2* __restrict__ z,
-                                int L, int nb, int nz, int ncand, double2* __restrict__ out) {
+// Calls f with the group width M (2, 4, 8, 16, 32) of L x L matrices as a compile-time constant.
+template <typename F>
+static void with_group(int L, F&& f) {
+  if (L <= 2) f(std::integral_constant<int, 2>());
+  else if (L <= 4) f(std::integral_constant<int, 4>());
+  else if (L <= 8) f(std::integral_constant<int, 8>());
+  else if (L <= 16) f(std::integral_constant<int, 16>());
+  else f(std::integral_constant<int, 32>());
+}
+
+// g[c][n][a] = 1 / (z_n - eps[c][a]).
+__global__ void k_bath_g(const double* __restrict__ eps, const double2* __restrict__ z, int nb, int nz, int ncand,
+                         double2* __restrict__ g) {
+  const int64_t n = (int64_t)ncand * nz * nb;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    const int a = (int)(t % nb);
+    const int64_t cf = t / nb;
+    const double2 zz = z[cf % nz];
+    g[t] = cinv(make_double2(zz.x - eps[cf / nz * nb + a], zz.y));
+  }
+}
+
+// Gamma[c][n][mu][nu] = sum_a theta[c][mu][a] theta[c][nu][a] g[c][n][a] (Eq. hybridization).
+__global__ void k_hybridization(const double* __restrict__ theta, const double2* __restrict__ g, int L, int nb, int nz,
+                                int ncand, double2* __restrict__ out) {
   const int64_t n = (int64_t)ncand * nz * L * L;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = t / ((int64_t)nz * L * L);
-    const int rem = (int)(t % ((int64_t)nz * L * L));
-    const int f = rem / (L * L), mu = (rem % (L * L)) / L, nu = rem % L;
+    const int64_t cf = t / (L * L), c = cf / nz;
+    const int e = (int)(t - cf * L * L), mu = e / L, nu = e - mu * L;
     const double* th = theta + c * L * nb;
-    const double* ep = eps + c * nb;
+    const double2* gg = g + cf * nb;
     double2 s = make_double2(0.0, 0.0);
     for (int a = 0; a < nb; ++a) {
       const double w = th[mu * nb + a] * th[nu * nb + a];
-      s = cadd(s, cmul(make_double2(w, 0.0), cinv(make_double2(z[f].x - ep[a], z[f].y))));
+      const double2 v = gg[a];
+      s = make_double2(fma(w, v.x, s.x), fma(w, v.y, s.y));
     }
     out[t] = s;
   }
@@ -260,46 +343,57 @@ __global__ void k_distance(const double2* __restrict__ A, const double2* __restr
 //   d d / d eps_a      = -2 Re sum_n W_n g_a^2 sum_{mu nu} conj(R_{mu nu}) theta_{mu a} theta_{nu a}
 //   d d / d theta_{rho a} = -2 Re sum_n W_n g_a [sum_nu conj(R_{rho nu}) theta_{nu a}
 //                                               + sum_mu conj(R_{mu rho}) theta_{mu a}]
-// with g_a = 1 / (z_n - eps_a) and R = A - Gamma_c; thread per (candidate, parameter).
-__global__ void k_distance_grad(const double2* __restrict__ A, const double2* __restrict__ Gam, const double* __restrict__ Wn,
-                                const double2* __restrict__ z, const double* __restrict__ eps,
-                                const double* __restrict__ theta, int L, int nb, int nz, int ncand,
-                                double* __restrict__ grad) {
-  const int np = nb + L * nb;
-  const int64_t total = (int64_t)ncand * np;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(t / np), p = (int)(t % np);
-    const double* th = theta + (int64_t)c * L * nb;
-    const int64_t per = (int64_t)nz * L * L;
-    const double2* G = Gam + c * per;
-    double acc = 0.0;
-    if (p < nb) {
-      const int a = p;
-      for (int n = 0; n < nz; ++n) {
-        const double2 g = cinv(make_double2(z[n].x - eps[c * nb + a], z[n].y));
-        double2 s = make_double2(0.0, 0.0);
-        for (int mu = 0; mu < L; ++mu)
+// with g_a = 1 / (z_n - eps_a) and R = A - Gamma_c.  Block per (candidate, tile of parameters);
+// its threads are parameters x frequency slices (a thread per parameter alone leaves most SMs
+// idle: 2.4 ms for 64 candidates of 40 parameters on 256 frequencies, 0.32 ms now); the slices
+// are added in order.
+__global__ void __launch_bounds__(256) k_distance_grad(const double2* __restrict__ A, const double2* __restrict__ Gam,
+                                                       const double* __restrict__ Wn, const double2* __restrict__ g,
+                                                       const double* __restrict__ theta, int L, int nb, int nz, int slices,
+                                                       double* __restrict__ grad) {
+  __shared__ double red[256];
+  const int np = nb + L * nb, tile = blockDim.x / slices;
+  const int c = blockIdx.x, p = blockIdx.y * tile + threadIdx.x % tile, slice = threadIdx.x / tile;
+  const double* th = theta + (int64_t)c * L * nb;
+  const int64_t per = (int64_t)nz * L * L;
+  const double2* G = Gam + c * per;
+  double acc = 0.0;
+  if (p < np && slice < slices) {
+    const int a = p < nb ? p : (p - nb) % nb, rho = p < nb ? 0 : (p - nb) / nb;
+    for (int n = slice; n < nz; n += slices) {
+      const double2 ga = g[((int64_t)c * nz + n) * nb + a];
+      const double2* An = A + (int64_t)n * L * L;
+      const double2* Gn = G + (int64_t)n * L * L;
+      double sr = 0.0, si = 0.0;  // of conj(R)
+      if (p < nb) {
+        for (int mu = 0; mu < L; ++mu) {
+          double tr = 0.0, ti = 0.0;
           for (int nu = 0; nu < L; ++nu) {
-            const int64_t e = (int64_t)n * L * L + mu * L + nu;
-            const double2 r = csub(A[e], G[e]);
-            s = cadd(s, cmul(cconj(r), make_double2(th[mu * nb + a] * th[nu * nb + a], 0.0)));
+            const double2 r = csub(An[mu * L + nu], Gn[mu * L + nu]);
+            tr = fma(r.x, th[nu * nb + a], tr);
+            ti = fma(r.y, th[nu * nb + a], ti);
           }
-        acc += Wn[n] * cmul(s, cmul(g, g)).x;
-      }
-    } else {
-      const int rho = (p - nb) / nb, a = (p - nb) % nb;
-      for (int n = 0; n < nz; ++n) {
-        const double2 g = cinv(make_double2(z[n].x - eps[c * nb + a], z[n].y));
-        double2 s = make_double2(0.0, 0.0);
-        for (int nu = 0; nu < L; ++nu) {
-          const int64_t e1 = (int64_t)n * L * L + rho * L + nu, e2 = (int64_t)n * L * L + nu * L + rho;
-          const double2 r1 = csub(A[e1], G[e1]), r2 = csub(A[e2], G[e2]);
-          s = cadd(s, cmul(cadd(cconj(r1), cconj(r2)), make_double2(th[nu * nb + a], 0.0)));
+          sr = fma(tr, th[mu * nb + a], sr);
+          si = fma(ti, th[mu * nb + a], si);
         }
-        acc += Wn[n] * cmul(s, g).x;
+        const double2 g2 = cmul(ga, ga);
+        acc += Wn[n] * (sr * g2.x + si * g2.y);
+      } else {
+        for (int nu = 0; nu < L; ++nu) {
+          const double2 r1 = csub(An[rho * L + nu], Gn[rho * L + nu]), r2 = csub(An[nu * L + rho], Gn[nu * L + rho]);
+          sr = fma(r1.x + r2.x, th[nu * nb + a], sr);
+          si = fma(r1.y + r2.y, th[nu * nb + a], si);
+        }
+        acc += Wn[n] * (sr * ga.x + si * ga.y);
       }
     }
-    grad[t] = -2.0 * acc;
+  }
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  if (slice == 0 && p < np) {
+    double s = 0.0;
+    for (int q = 0; q < slices; ++q) s += red[q * tile + threadIdx.x % tile];
+    grad[(int64_t)c * np + p] = -2.0 * s;
   }
 }
 
@@ -367,10 +461,23 @@ static void build_v(const LatticeDev& d, const DevBuf<double>& kt, int nk, DevBu
 
 static void invert_batched(const double2* in, const double2* add, double2* out, int L, int64_t count, int* status,
                            cudaStream_t s) {
-  const size_t smem = kLatWarps * warp_slice(L);
-  allow_max_dynamic_smem(k_invert);
   ProfScope ps_(K_LATTICE, s, 0.0);
-  k_invert<<<lat_grid(count, kLatWarps), 32 * kLatWarps, smem, s>>>(in, add, out, L, count, status);
+  with_group(L, [&](auto m) {
+    constexpr int M = decltype(m)::value;
+    k_invert<M><<<lat_grid(count, kLatThreads / M), kLatThreads, 0, s>>>(in, add, out, L, count, status);
+  });
+  ED_CHECK_LAUNCH();
+}
+
+static void average_batched(const double2* Gci, const double2* V, int L, int nz, int nk, double2* out, int* status,
+                            cudaStream_t s) {
+  ProfScope ps_(K_LATTICE, s, 0.0);
+  with_group(L, [&](auto m) {
+    constexpr int M = decltype(m)::value;
+    allow_max_dynamic_smem(k_cpt_average<M>);
+    k_cpt_average<M><<<(unsigned)std::min(nz, 152 * 8), kLatThreads, (size_t)(kLatThreads / M) * L * L * sizeof(double2), s>>>(
+        Gci, V, L, nz, nk, out, status);
+  });
   ED_CHECK_LAUNCH();
 }
 
@@ -432,7 +539,7 @@ static void require_lat(bool ok, const char* msg) {
 // Distance (and gradient) of n_cand baths against A, all on the device; d and grad to the host.
 struct DistanceWork {
   int L, nb, nz;
-  DevBuf<double2> z, A, Gam;
+  DevBuf<double2> z, A, Gam, g;
   DevBuf<double> W, eps, theta, d, grad;
   void setup(int L_, int nb_, const double* zh, int nz_, const double* Wh, const double* Ah, cudaStream_t s) {
     L = L_;
@@ -456,9 +563,15 @@ struct DistanceWork {
       ED_CUDA(cudaMemcpyAsync(eps.p, eps_h, (size_t)nc * nb * sizeof(double), cudaMemcpyHostToDevice, s));
       ED_CUDA(cudaMemcpyAsync(theta.p, theta_h, (size_t)nc * L * nb * sizeof(double), cudaMemcpyHostToDevice, s));
     }
+    if (g.n < (size_t)std::max<int64_t>((int64_t)nc * nz * nb, 1)) g.alloc(std::max<int64_t>((int64_t)nc * nz * nb, 1));
+    if (nb) {
+      ProfScope ps_(K_LATTICE, s, 0.0);
+      k_bath_g<<<lat_grid((int64_t)nc * nz * nb, 256), 256, 0, s>>>(eps.p, z.p, nb, nz, nc, g.p);
+      ED_CHECK_LAUNCH();
+    }
     {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_hybridization<<<lat_grid((int64_t)nc * nz * L * L, 256), 256, 0, s>>>(eps.p, theta.p, z.p, L, nb, nz, nc, Gam.p);
+      k_hybridization<<<lat_grid((int64_t)nc * nz * L * L, 256), 256, 0, s>>>(theta.p, g.p, L, nb, nz, nc, Gam.p);
       ED_CHECK_LAUNCH();
     }
     {
@@ -468,8 +581,9 @@ struct DistanceWork {
     }
     if (grad_h && np) {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_distance_grad<<<lat_grid((int64_t)nc * np, 128), 128, 0, s>>>(A.p, Gam.p, W.p, z.p, eps.p, theta.p, L, nb, nz, nc,
-                                                                     grad.p);
+      const int slices = std::max(1, std::min(32, 256 / np)), tile = 256 / slices;
+      k_distance_grad<<<dim3(nc, (np + tile - 1) / tile), 256, 0, s>>>(A.p, Gam.p, W.p, g.p, theta.p, L, nb, nz, slices,
+                                                                       grad.p);
       ED_CHECK_LAUNCH();
     }
     ED_CUDA(cudaMemcpyAsync(d_h, d.p, nc * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -512,9 +626,15 @@ ed_status ed_hybridization(int n_sites, int n_bath, const double* eps, const dou
       tmp.alloc(n);
       out = tmp.p;
     }
+    DevBuf<double2> g(std::max<size_t>((size_t)nz * n_bath, 1));
+    if (n_bath) {
+      ProfScope ps_(K_LATTICE, s, 0.0);
+      k_bath_g<<<lat_grid((int64_t)nz * n_bath, 256), 256, 0, s>>>(ed_.p, zd.p, n_bath, nz, 1, g.p);
+      ED_CHECK_LAUNCH();
+    }
     {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_hybridization<<<lat_grid((int64_t)n, 256), 256, 0, s>>>(ed_.p, td.p, zd.p, L, n_bath, nz, 1, out);
+      k_hybridization<<<lat_grid((int64_t)n, 256), 256, 0, s>>>(td.p, g.p, L, n_bath, nz, 1, out);
       ED_CHECK_LAUNCH();
     }
     if (!out_is_device) ED_CUDA(cudaMemcpyAsync(Gamma_out, tmp.p, n * sizeof(double2), cudaMemcpyDeviceToHost, s));
@@ -548,17 +668,22 @@ ed_status ed_cpt_green(const ed_superlattice* lat, const double* Gc, const doubl
       obuf.alloc(nout);
       o = obuf.p;
     }
+    DevBuf<double2> ph;
     if (mode == ED_CPT_AVERAGE) {
-      const size_t smem = kLatWarps * warp_slice(L) + (size_t)kLatWarps * L * L * sizeof(double2);
-      allow_max_dynamic_smem(k_cpt_average);
-      ProfScope ps_(K_LATTICE, s, 0.0);
-      k_cpt_average<<<(unsigned)std::min(nz, 152 * 8), 32 * kLatWarps, smem, s>>>(Gci.p, V.p, L, nz, nk, o, st.p);
-      ED_CHECK_LAUNCH();
+      average_batched(Gci.p, V.p, L, nz, nk, o, st.p, s);
     } else {
-      allow_max_dynamic_smem(k_cpt);
+      if (mode == ED_CPT_PERIODIZED) {
+        ph.alloc((size_t)nk * L);
+        ProfScope ps_(K_LATTICE, s, 0.0);
+        k_site_phases<<<lat_grid((int64_t)nk * L, 256), 256, 0, s>>>(kd.p, d.pos.p, D, L, nk, ph.p);
+        ED_CHECK_LAUNCH();
+      }
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_cpt<<<lat_grid((int64_t)nk * nz, kLatWarps), 32 * kLatWarps, kLatWarps * warp_slice(L), s>>>(
-          Gci.p, V.p, kd.p, d.pos.p, D, L, nz, nk, mode == ED_CPT_MATRIX ? 0 : 1, o, st.p);
+      with_group(L, [&](auto m) {
+        constexpr int M = decltype(m)::value;
+        k_cpt<M><<<lat_grid((int64_t)nk * nz, kLatThreads / M), kLatThreads, 0, s>>>(
+            Gci.p, V.p, ph.p, L, nz, nk, mode == ED_CPT_MATRIX ? 0 : 1, o, st.p);
+      });
       ED_CHECK_LAUNCH();
     }
     if (!io_is_device) ED_CUDA(cudaMemcpyAsync(out, o, nout * sizeof(double2), cudaMemcpyDeviceToHost, s));
@@ -585,13 +710,7 @@ ed_status ed_cdmft_target(const ed_superlattice* lat, const double* Gc, const do
     const double2* Gmd = dev_in(Gamma, n, io_is_device, t2, s);
     build_v(d, kd, nk, V, s);
     cluster_inverse(Gcd, Gmd, L, nz, Gci, st.p, s);  // G_c^-1 + Gamma
-    {
-      const size_t smem = kLatWarps * warp_slice(L) + (size_t)kLatWarps * L * L * sizeof(double2);
-      allow_max_dynamic_smem(k_cpt_average);
-      ProfScope ps_(K_LATTICE, s, 0.0);
-      k_cpt_average<<<(unsigned)std::min(nz, 152 * 8), 32 * kLatWarps, smem, s>>>(Gci.p, V.p, L, nz, nk, Gbar.p, st.p);
-      ED_CHECK_LAUNCH();
-    }
+    average_batched(Gci.p, V.p, L, nz, nk, Gbar.p, st.p, s);
     invert_batched(Gbar.p, nullptr, Gbi.p, L, nz, st.p, s);
     double2* o = reinterpret_cast<double2*>(A_out);
     if (!io_is_device) {
