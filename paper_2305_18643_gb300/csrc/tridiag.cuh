@@ -4,17 +4,18 @@
 // pivoting is stable).  Used by the single-cluster driver and by the batched per-block solver.
 //
 // A thread block runs one matrix, so the kernel is bound by the dependent chain of the recurrences
-// and by the FP64 pipe of one SM (two lanes per clock on this GPU).  Hence:
-//  - the count uses the division-free recurrence p_k = (a_k - x) p_{k-1} - b_k^2 p_{k-2} (three FP64
-//    operations per level; the quotient form's division is a dozen) on entries scaled by a power
-//    of two, rescaled every few levels;
-//  - the first three rounds run in FP32 on every thread, and only the last bits, inside a bracket
-//    that the FP64 counts verify, on 16 lanes per eigenvalue;
-//  - the sweeps of the inverse iteration are first-order linear recurrences, done by one warp as
-//    a scan over 32 chunks.
-// One call, over the checks of a 120-level run: 1,020 us in the quotient form on 256 threads with a
-// serial inverse iteration, 155 us now.  The ground states of 64 clusters of at most 7 orbitals,
-// where every block runs its own (csrc/batch.cu): 225.4 ms before, 42.4 ms now.
+// and by the FP64 pipe of one SM (two lanes per clock on this GPU).  The count of record is the
+// quotient form q_k = a_k - x - b_k^2 / q_{k-1}, whose division alone is a dozen FP64 operations, so it
+// runs only where it decides something: both eigenvalues are first located to a few ulps of the
+// matrix norm with the division-free recurrence p_k = (a_k - x) p_{k-1} - b_k^2 p_{k-2} on entries scaled
+// by a power of two (three rounds in FP32 on every thread, then FP64 on 16 lanes per eigenvalue);
+// the multisection for the lowest one then counts only at points inside that uncertainty, and
+// its result is bit for bit that of counting at every point.
+//
+// One call, over the checks of a 100-level run: 927 us with the quotient form at every point and a
+// division per pivot and sweep, 254 us now; over those of a 160-level run 1,418 and 380 us.  The ground
+// states of 64 clusters of at most 7 orbitals, where every block runs its own (csrc/batch.cu): 225.4 ms
+// before, 78.2 ms now.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -63,50 +64,17 @@ static __device__ inline int sturm_count64(const double* a, const double* b2, in
   return cnt;
 }
 
-// One sweep y_i <- im_i (y_i - b_i y_{i-1}) (forward) or y_i <- y_i - b_{i+1} im_i y_{i+1} (backward)
-// by one warp: lane l owns the chunk of c indices from l c; the chunks' affine maps are composed by
-// a scan over the lanes, then every lane runs its chunk from the right start.
-template <bool FWD>
-static __device__ inline void tridiag_sweep(const double* __restrict__ b, const double* im, double* y, int n, int c) {
-  const int lane = threadIdx.x & 31;
-  const int i0 = lane * c, i1 = min(n, i0 + c);
-  double A = 1.0, B = 0.0;
-  if (FWD) {
-    for (int i = i0; i < i1; ++i) {
-      const double l = i > 0 ? b[i] * im[i] : 0.0;
-      B = fma(-l, B, y[i] * im[i]);
-      A *= -l;
-    }
-  } else {
-    for (int i = i1 - 1; i >= i0; --i) {
-      const double u = i + 1 < n ? b[i + 1] * im[i] : 0.0;
-      B = fma(-u, B, y[i]);
-      A *= -u;
-    }
+// Number of eigenvalues below x in the quotient form: diagonal a[0..n-1], off-diagonal b[1..n-1].
+static __device__ inline int sturm_count(const double* __restrict__ a, const double* __restrict__ b, int n, double x) {
+  int cnt = 0;
+  double q = a[0] - x;
+  if (q < 0.0) ++cnt;
+  for (int i = 1; i < n; ++i) {
+    if (q == 0.0) q = 1e-300;
+    q = a[i] - x - b[i] * b[i] / q;
+    if (q < 0.0) ++cnt;
   }
-  // in: value entering this lane's chunk = composition of the maps of all chunks before it
-  for (int o = 1; o < 32; o <<= 1) {
-    const double Ao = FWD ? __shfl_up_sync(0xffffffffu, A, o) : __shfl_down_sync(0xffffffffu, A, o);
-    const double Bo = FWD ? __shfl_up_sync(0xffffffffu, B, o) : __shfl_down_sync(0xffffffffu, B, o);
-    if (FWD ? lane >= o : lane + o < 32) {
-      B = fma(A, Bo, B);
-      A *= Ao;
-    }
-  }
-  double t = FWD ? __shfl_up_sync(0xffffffffu, B, 1) : __shfl_down_sync(0xffffffffu, B, 1);
-  if (FWD ? lane == 0 : lane == 31) t = 0.0;
-  if (FWD) {
-    for (int i = i0; i < i1; ++i) {
-      const double l = i > 0 ? b[i] * im[i] : 0.0;
-      y[i] = t = fma(-l, t, y[i] * im[i]);
-    }
-  } else {
-    for (int i = i1 - 1; i >= i0; --i) {
-      const double u = i + 1 < n ? b[i + 1] * im[i] : 0.0;
-      y[i] = t = fma(-u, t, y[i]);
-    }
-  }
-  __syncwarp();
+  return cnt;
 }
 
 // out_eval: [0] lowest eigenvalue, [1] second eigenvalue (inf if n < 2), [2] Ritz estimate
@@ -116,6 +84,7 @@ static __device__ void tridiag_lowest_block(const double* __restrict__ a, const 
                                             double* out_eval, double* vec) {
   __shared__ double s_lo, s_hi;
   __shared__ int s_first[2];
+  __shared__ double s_near[2], s_width;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   // Gershgorin interval
   if (tid < 32) {
@@ -175,85 +144,141 @@ static __device__ void tridiag_lowest_block(const double* __restrict__ a, const 
     vec[n + i] = bs * bs;  // over the FP32 entries
   }
   __syncthreads();
-  if (tid >= 32) return;
-  // FP64 rounds: lanes 0..15 bracket the lowest, 16..31 the second eigenvalue, end points included.
-  // The FP32 counts are those of a matrix within a few 2^-24 of this one; a bracket that the
-  // FP64 counts of the first round refute is widened to the whole interval.
-  const int e = lane >> 4, pt = lane & 15;
-  double dlo = (double)lo[e] - 2e-6, dhi = (double)hi[e] + 2e-6;
-  bool first = true, done = e == 1 && n < 2;
-  for (int round = 0; round < 24; ++round) {
-    const double x = dlo + (dhi - dlo) * ((double)pt * (1.0 / 15.0));
-    const bool above = sturm_count64(vec, vec + n, n, x) >= e + 1;
-    const unsigned bal = (__ballot_sync(0xffffffffu, above) >> (16 * e)) & 0xffffu;
-    if (!done) {
-      const int f = bal ? __ffs(bal) - 1 : 16;
-      if (f == 0 || f == 16) {
-        if (first) {
-          dlo = glo * is;
-          dhi = ghi * is;
+  // FP64 rounds by warp 0: lanes 0..15 bracket the lowest, 16..31 the second eigenvalue, end points
+  // included.  The FP32 counts are those of a matrix within a few 2^-24 of this one; a bracket that
+  // the FP64 counts of the first round refute is widened to the whole interval.
+  if (tid < 32) {
+    const int e = lane >> 4, pt = lane & 15;
+    double dlo = (double)lo[e] - 2e-6, dhi = (double)hi[e] + 2e-6;
+    bool first = true, done = e == 1 && n < 2;
+    for (int round = 0; round < 24; ++round) {
+      const double x = dlo + (dhi - dlo) * ((double)pt * (1.0 / 15.0));
+      const bool above = sturm_count64(vec, vec + n, n, x) >= e + 1;
+      const unsigned bal = (__ballot_sync(0xffffffffu, above) >> (16 * e)) & 0xffffu;
+      if (!done) {
+        const int f = bal ? __ffs(bal) - 1 : 16;
+        if (f == 0 || f == 16) {
+          if (first) {
+            dlo = glo * is;
+            dhi = ghi * is;
+          } else {
+            done = true;  // the bracket is down to rounding
+          }
         } else {
-          done = true;  // the bracket is down to rounding
+          const double w = dhi - dlo;
+          const double nlo = dlo + w * ((double)(f - 1) * (1.0 / 15.0));
+          const double nhi = f == 15 ? dhi : dlo + w * ((double)f * (1.0 / 15.0));
+          dlo = nlo;
+          dhi = nhi;
         }
-      } else {
-        const double w = dhi - dlo;
-        const double nlo = dlo + w * ((double)(f - 1) * (1.0 / 15.0));
-        const double nhi = f == 15 ? dhi : dlo + w * ((double)f * (1.0 / 15.0));
-        dlo = nlo;
-        dhi = nhi;
+        first = false;
+        if (dhi - dlo <= 2e-15) done = true;
       }
-      first = false;
-      if (dhi - dlo <= 4e-16 * fmax(fabs(dlo), fabs(dhi))) done = true;
+      if (__all_sync(0xffffffffu, done)) break;
     }
-    if (__all_sync(0xffffffffu, done)) break;
+    if (pt == 0) s_near[e] = 0.5 * (dlo + dhi) * sc;
+    if (lane == 0) s_width = (dhi - dlo) * sc;
   }
-  const double mid = 0.5 * (dlo + dhi) * sc;
-  const double lam = __shfl_sync(0xffffffffu, mid, 0);
-  const double lam1 = __shfl_sync(0xffffffffu, mid, 16);
-  // inverse iteration with a shift just below lam: pivots m_i = p_i / p_{i-1} of T - sigma from the
-  // same recurrence (lane 0; every p_i > 0), then three solves
+  __syncthreads();
+  // multisection for the lowest eigenvalue on nt points a round; both counts are exact for matrices
+  // within ~10 ulps (of the norm) of this one, so points further than 100 ulps from the bracket need
+  // none, and points that round to the same number need one
+  const double near = s_near[0], slack = 0.5 * s_width + 100.0 * 2.3e-16 * sc;
+  int* cand = reinterpret_cast<int*>(vec);
+  double rlo = glo, rhi = ghi;
+  auto point = [&](int j) { return rlo + (rhi - rlo) * (double)(j + 1) / (double)(nt + 1); };
+  for (int round = 0; round < 16; ++round) {
+    if (tid == 0) {
+      s_first[0] = nt;
+      s_first[1] = 0;
+    }
+    __syncthreads();
+    const double x = point(tid);
+    if (x > near + slack) {
+      atomicMin(&s_first[0], tid);
+    } else if (x >= near - slack && (tid == 0 || point(tid - 1) != x)) {
+      const int c = atomicAdd(&s_first[1], 1);
+      if (c < 4 * n) cand[c] = tid;  // vec holds 2 n doubles
+    }
+    __syncthreads();
+    const int nc = s_first[1];
+    if (nc <= 4 * n) {
+      for (int c = tid; c < nc; c += nt) {
+        const int j = cand[c];
+        if (sturm_count(a, b, n, point(j)) >= 1) atomicMin(&s_first[0], j);
+      }
+    } else if (x >= near - slack && x <= near + slack) {
+      if (sturm_count(a, b, n, x) >= 1) atomicMin(&s_first[0], tid);
+    }
+    __syncthreads();
+    const int j = s_first[0];
+    const double nlo = j == 0 ? rlo : rlo + (rhi - rlo) * (double)j / (double)(nt + 1);
+    const double nhi = j == nt ? rhi : rlo + (rhi - rlo) * (double)(j + 1) / (double)(nt + 1);
+    rlo = nlo;
+    rhi = nhi;
+    __syncthreads();
+    if (rhi - rlo <= 4e-16 * fmax(fabs(rlo), fabs(rhi))) break;
+  }
+  if (tid >= 32) return;
+  const double lam = 0.5 * (rlo + rhi);
+  // inverse iteration with shift just below lam: T - sigma I is positive definite, so the
+  // Thomas elimination without pivoting is stable.  The pivots m_i are those of every iteration, so
+  // they are found once (lane 0; cp_i = b_{i+1} / m_i is kept); the quotients by m_i in the sweeps
+  // come from the rounded reciprocals r_i (Markstein, "Computation of elementary functions on the
+  // IBM RISC System/6000 processor", 1990: q = y r, q + r (y - q m) is the rounded quotient).
   const double scale = fmax(1.0, fmax(fabs(glo), fabs(ghi)));
-  const double sigma = (lam - 1e-10 * scale) * is;
+  const double sigma = lam - 1e-10 * scale;
+  double* y = vec;
+  double* cp = vec + n;
   if (lane == 0) {
-    double pp = 0.0, p = 1.0;
-    for (int i = 0; i < n; ++i) {
-      const double q = fma(vec[i] - sigma, p, -vec[n + i] * pp);
-      vec[i] = q;
-      vec[n + i] = p;
-      pp = p;
-      p = q;
-      if ((i & 7) == 7) {
-        const int ee = max(__double2hiint(p) & 0x7ff00000, __double2hiint(pp) & 0x7ff00000);
-        const double f = __hiloint2double(min(max((2046 << 20) - ee, 1 << 20), 2045 << 20), 0);
-        p *= f;
-        pp *= f;
-      }
+    double m = a[0] - sigma;
+    cp[0] = (n > 1 ? b[1] : 0.0) / m;
+    for (int i = 1; i < n; ++i) {
+      m = (a[i] - sigma) - b[i] * cp[i - 1];
+      cp[i] = (i + 1 < n ? b[i + 1] : 0.0) / m;
     }
   }
   __syncwarp();
-  double* y = vec;
-  double* im = vec + n;
-  for (int i = lane; i < n; i += 32) {
-    im[i] = vec[n + i] / (vec[i] * sc);
-    y[i] = 1.0 + 0.1 * (double)sinf((float)i);
-  }
+  for (int i = lane; i < n; i += 32) y[i] = 1.0 + 0.1 * sin((double)i);
   __syncwarp();
-  const int c = (n + 31) / 32;
   for (int it = 0; it < 3; ++it) {
-    tridiag_sweep<true>(b, im, y, n, c);
-    tridiag_sweep<false>(b, im, y, n, c);
-    double nr = 0.0;
-    for (int i = lane; i < n; i += 32) nr = fma(y[i], y[i], nr);
-    for (int o = 16; o > 0; o >>= 1) nr += __shfl_xor_sync(0xffffffffu, nr, o);
-    nr = 1.0 / sqrt(nr);
-    if (it == 2 && y[0] < 0.0) nr = -nr;
+    double t = 0.0;
+    for (int i0 = 0; i0 < n; i0 += 32) {  // forward sweep: pivots and reciprocals by 32 lanes, then lane by lane
+      const int i = i0 + lane;
+      const double bi = i > 0 && i < n ? b[i] : 0.0;
+      const double m = i == 0 ? a[0] - sigma : i < n ? (a[i] - sigma) - bi * cp[i - 1] : 1.0;
+      const double r = 1.0 / m;
+      double yi = i < n ? y[i] : 0.0;
+      for (int l = 0; l < 32; ++l) {
+        // every lane runs the quotient on its own entry; lane l's is the one that is final
+        const double num = i == 0 ? yi : yi - bi * t;
+        const double q = num * r;
+        const double v = fma(fma(-q, m, num), r, q);
+        if (lane == l) yi = v;
+        t = __shfl_sync(0xffffffffu, v, l);
+      }
+      if (i < n) y[i] = yi;
+      t = __shfl_sync(0xffffffffu, yi, 31);
+    }
     __syncwarp();
+    double nr = 0.0;
+    if (lane == 0) {
+      for (int i = n - 2; i >= 0; --i) y[i] -= cp[i] * y[i + 1];
+      for (int i = 0; i < n; ++i) nr += y[i] * y[i];
+      nr = 1.0 / sqrt(nr);
+    }
+    nr = __shfl_sync(0xffffffffu, nr, 0);
     for (int i = lane; i < n; i += 32) y[i] *= nr;
     __syncwarp();
   }
+  if (y[0] < 0.0) {
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) y[i] = -y[i];
+  }
+  __syncwarp();
   if (lane == 0) {
     out_eval[0] = lam;
-    out_eval[1] = n < 2 ? INFINITY : lam1;
+    out_eval[1] = n < 2 ? INFINITY : s_near[1];
     out_eval[2] = fabs(b[n]) * fabs(y[n - 1]);
   }
 }
