@@ -22,6 +22,7 @@
 #include <numeric>
 #include <tuple>
 
+#include "cf.cuh"
 #include "ed_common.cuh"
 #include "tridiag.cuh"
 
@@ -1010,14 +1011,17 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
 }
 
 // -------------------------------------------------------------------------------- evaluation on the grid
-__global__ void k_bcf_eval(const BRun* __restrict__ R, int nruns, const BCluster* __restrict__ C,
-                           const double2* __restrict__ z, int nz, double2* __restrict__ out) {
+constexpr int kEvalThreads = 128;
+__global__ void __launch_bounds__(kEvalThreads) k_bcf_eval(const BRun* __restrict__ R, int nruns,
+                                                           const BCluster* __restrict__ C, const double2* __restrict__ z,
+                                                           int nz, double2* __restrict__ out) {
+  __shared__ double2 sm[kCfChunk];
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= nz) return;
   for (int q = blockIdx.y; q < nruns; q += gridDim.y) {  // grid.y is capped at 65535
     const BRun& r = R[q];
-    out[(int64_t)q * nz + k] =
-        b_cf_eval(r.alpha, r.beta, r.nsteps, r.b0sq, z[k], C[r.cluster].E0, r.part == 0 ? -1.0 : 1.0);
+    const double2 g = cf_eval_block(r.alpha, r.beta, r.nsteps, r.b0sq, z[min(k, nz - 1)], C[r.cluster].E0,
+                                    r.part == 0 ? -1.0 : 1.0, sm, k < nz);
+    if (k < nz) out[(int64_t)q * nz + k] = g;
   }
 }
 
@@ -1467,7 +1471,7 @@ void batch_solve(const ed_cluster_desc* descs, int n, int precision, const doubl
       run_batch_kernels<float>(cfg.first, cfg.second, dC.p, dCo.p, n, dT.p, dR.p, dRo.p, nblock_runs, nruns, dG.p, ngroups, dQ.p, w, blocks,
                                dz.p, nz, gtol, do_gf, s, false);
     if (gf) {
-      k_bcf_eval<<<dim3((nz + 255) / 256, std::min(nruns, 32768)), 256, 0, s>>>(dR.p, nruns, dC.p, dz.p, nz, Gk);
+      k_bcf_eval<<<dim3((nz + kEvalThreads - 1) / kEvalThreads, std::min(nruns, 32768)), kEvalThreads, 0, s>>>(dR.p, nruns, dC.p, dz.p, nz, Gk);
       ED_CHECK_LAUNCH();
       k_bcombine<<<dim3(64, std::min(n, 32768)), 256, 0, s>>>(dC.p, n, dBase.p, dgoff.p, Gk, nz, G_dev_out);
       ED_CHECK_LAUNCH();

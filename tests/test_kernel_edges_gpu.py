@@ -92,3 +92,16 @@ def test_distance_gradient_tiles(L, nb, nc):
     ref = np.concatenate([ge, gt.reshape(nc, -1)], axis=1)
     assert np.abs(d - d_ref).max() <= 1e-12 * np.abs(d_ref).max()
     assert np.abs(grad - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+# Continued fractions: thread blocks of 64 and 128 frequencies, levels staged 128 at a time (300-state
+# sectors run past their dimension), checks on every second frequency from 2,048 on.
+@pytest.mark.parametrize("nz", [1, 63, 65, 129, 2100])
+def test_continued_fraction_grid_edges(nz):
+    c = W.random_cluster(np.random.default_rng(3), 6, 0, 3, 3)
+    om = np.linspace(-6.0, 6.0, nz)
+    ref = O.green_exact(_model(c), 3, 3, om + 0.05j)[0]
+    with ed.Cluster(c, seed=5) as cl:
+        assert np.abs(cl.green(om, 0.05) - ref).max() <= 1e-8
+    G = ed.ed_batch_solve([c], omega=om, eta=0.05, seed=5)[4][0]
+    assert np.abs(G[0] - ref).max() <= 1e-8 and np.abs(G[1] - ref).max() <= 1e-8
