@@ -231,6 +231,29 @@ struct BPart3<float> {
   __device__ double get(int i) const { return (double)s[i] - (double)k[i]; }
 };
 
+// acc + sum_{k < cnt} (+-val) X[col stride] over the slot-major entries p[k step], in the order of k.
+// Four entries, values and operands are loaded ahead of their multiply-adds: a warp has few others
+// to hide behind, and one hop at a time costs the latency of two dependent loads and an FMA.
+template <typename T>
+__device__ __forceinline__ T add_hops(T acc, const uint32_t* __restrict__ p, int64_t step, int cnt,
+                                      const T* __restrict__ val, const T* X, int64_t stride) {
+  for (int k = 0; k < cnt; k += 4) {
+    uint32_t e[4];
+    T v[4], x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) e[i] = k + i < cnt ? p[(int64_t)(k + i) * step] : 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[i] = val[ent_vidx(e[i])];
+      x[i] = X[(int64_t)ent_col(e[i]) * stride];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (k + i < cnt) acc += (ent_neg(e[i]) ? -v[i] : v[i]) * x[i];
+  }
+  return acc;
+}
+
 // W = H X - bcoef * W (in place; W may hold x_prev), with <x,w>, <w,w>, <x,x> returned to every
 // thread.  mode 0: element-strided (consecutive threads take consecutive elements); mode 1: one
 // warp per row (warp-uniform up-spin entries, lanes over the columns).
@@ -256,19 +279,8 @@ __device__ void block_hx(const BTable& tu, const BTable& td, const T* sval, cons
     }
     const T x = X[o];
     T acc = diag * x;
-    const T* xr = X + u * dd;
-    const int nd = td.cnt[d];
-    for (int k = 0; k < nd; ++k) {
-      const uint32_t e = td.ell[(int64_t)k * dd + d];
-      const T v = sval[ent_vidx(e)];
-      acc += (ent_neg(e) ? -v : v) * xr[ent_col(e)];
-    }
-    const int nu = tu.cnt[u];
-    for (int k = 0; k < nu; ++k) {
-      const uint32_t e = tu.ell[(int64_t)k * du + u];
-      const T v = sval[ent_vidx(e)];
-      acc += (ent_neg(e) ? -v : v) * X[(int64_t)ent_col(e) * dd + d];
-    }
+    acc = add_hops<T>(acc, td.ell + d, dd, td.cnt[d], sval, X + u * dd, 1);
+    acc = add_hops<T>(acc, tu.ell + u, du, tu.cnt[u], sval, X + d, dd);
     const T w = acc - bcoef * W[o];
     W[o] = w;
     part.add(x, w);
@@ -627,6 +639,7 @@ __global__ void k_batch_gs(BCluster* __restrict__ C, const int* __restrict__ ord
 struct CFShared {
   BlockShared bs;
   double2 prev[4][64];
+  CfForward st[4][64];
   double red12[12][32];
   double bcast12[12];
   double maxdiff;
@@ -637,38 +650,42 @@ struct CFShared {
   int flag;
 };
 
-__device__ __forceinline__ double2 b_cf_eval(const double* __restrict__ a, const double* __restrict__ b, int m,
-                                             double b0sq, double2 z, double E0, double s) {
-  if (m <= 0) return make_double2(0.0, 0.0);
-  double dr = z.x + s * (a[m - 1] - E0), di = z.y;
-  for (int k = m - 2; k >= 0; --k) {
-    const double bb = b[k + 1];
-    const double q = bb * bb / (dr * dr + di * di);
-    dr = z.x + s * (a[k] - E0) - q * dr;
-    di = z.y + q * di;
-  }
-  const double q = b0sq / (dr * dr + di * di);
-  return make_double2(q * dr, -q * di);
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// W = H X - bcoef W over a sector by one warp (lanes over elements, fixed butterfly sums), with
-// <x,w>, <w,w>, <x,x> returned to every lane.  Hopping values and U come from the cluster's
-// parameters in global memory (cached).
+// Diagonal of H over a sector, D[u][d], by one warp (it serves every level of the run).
 template <typename T>
-__device__ void warp_hx(const BTable& tu, const BTable& td, const HopParams& hp, const T* X, T* W, T bcoef,
-                        double& sxw, double& sww, double& sxx) {
-  const int lane = threadIdx.x & 31;
-  const int64_t du = tu.dim, dd = td.dim;
+__device__ void warp_diag(const BTable& tu, const BTable& td, const HopParams& hp, T* D) {
+  const int64_t dd = td.dim, n = tu.dim * dd;
   const T* eu = BP<T>::e(tu);
   const T* ed = BP<T>::e(td);
   const T u0 = (T)hp.u0;
   const bool uni = hp.uniform_u != 0;
-  const uint32_t umask = hp.umask;
+  for (int64_t o = threadIdx.x & 31; o < n; o += 32) {
+    const int64_t u = o / dd, d = o - u * dd;
+    T diag = eu[u] + ed[d];
+    uint32_t dbl = tu.basis[u] & td.basis[d] & hp.umask;
+    if (uni) {
+      diag += u0 * (T)__popc(dbl);
+    } else {
+      while (dbl) {
+        diag += BP<T>::U(hp, __ffs(dbl) - 1);
+        dbl &= dbl - 1u;
+      }
+    }
+    D[o] = diag;
+  }
+}
+
+// W = H X - bcoef W over a sector by one warp (lanes over elements, fixed butterfly sums), with
+// <x,w>, <w,w>, <x,x> returned to every lane.  D: the diagonal; val: the hopping values.
+template <typename T>
+__device__ void warp_hx(const BTable& tu, const BTable& td, const T* D, const T* __restrict__ val, const T* X, T* W, T bcoef,
+                        double& sxw, double& sww, double& sxx) {
+  const int lane = threadIdx.x & 31;
+  const int64_t du = tu.dim, dd = td.dim;
   BPart3<T> part;
   const int64_t su = 32 / dd, sd = 32 - su * dd;
   int64_t u = lane / dd, d = lane - u * dd;
@@ -679,32 +696,10 @@ __device__ void warp_hx(const BTable& tu, const BTable& td, const HopParams& hp,
       if (u >= du) break;
     }
     const int64_t o = u * dd + d;
-    const uint32_t bu = tu.basis[u], bd = td.basis[d];
-    T diag = eu[u] + ed[d];
-    uint32_t dbl = bu & bd & umask;
-    if (uni) {
-      diag += u0 * (T)__popc(dbl);
-    } else {
-      while (dbl) {
-        diag += BP<T>::U(hp, __ffs(dbl) - 1);
-        dbl &= dbl - 1u;
-      }
-    }
     const T x = X[o];
-    T acc = diag * x;
-    const T* xr = X + u * dd;
-    const int nd = td.cnt[d];
-    for (int k = 0; k < nd; ++k) {
-      const uint32_t e = td.ell[(int64_t)k * dd + d];
-      const T v = BP<T>::val(hp, ent_vidx(e));
-      acc += (ent_neg(e) ? -v : v) * xr[ent_col(e)];
-    }
-    const int nu = tu.cnt[u];
-    for (int k = 0; k < nu; ++k) {
-      const uint32_t e = tu.ell[(int64_t)k * du + u];
-      const T v = BP<T>::val(hp, ent_vidx(e));
-      acc += (ent_neg(e) ? -v : v) * X[(int64_t)ent_col(e) * dd + d];
-    }
+    T acc = D[o] * x;
+    acc = add_hops<T>(acc, td.ell + d, dd, td.cnt[d], val, X + u * dd, 1);
+    acc = add_hops<T>(acc, tu.ell + u, du, tu.cnt[u], val, X + d, dd);
     const T w = acc - bcoef * W[o];
     W[o] = w;
     part.add(x, w);
@@ -714,10 +709,22 @@ __device__ void warp_hx(const BTable& tu, const BTable& td, const HopParams& hp,
   sxx = warp_sum(part.get(2));
 }
 
+// The convergence check of one frequency (cf.cuh, forward form): advances its state over the levels
+// [m0, m) of the coefficients a, b.
+__device__ __forceinline__ double2 cf_advance(CfForward& st, const double* __restrict__ a, const double* __restrict__ b,
+                                              int m0, int m, double b0sq, double2 z, double E0, double s) {
+  for (int n = m0; n < m; ++n) {
+    st.level(make_double2(s * (a[n] - E0), n == 0 ? -1.0 : b[n] * b[n]), z);
+    if ((n & 7) == 7) st.rescale();
+  }
+  st.rescale();
+  return st.value(b0sq);
+}
+
 // One continued fraction run by one warp: the same steps, check schedule and stopping rule as
 // the block-level run of k_batch_cf.
 template <typename T>
-__device__ void warp_cf_run(BRun& r, const BCluster& c, const BTable* tabs, T* V0, T* V1, const double2* z, int nz,
+__device__ void warp_cf_run(BRun& r, const BCluster& c, const BTable* tabs, T* V0, T* V1, T* D, const double2* z, int nz,
                             double tol) {
   const int lane = threadIdx.x & 31;
   const int zstride = max(1, (nz + 63) / 64);
@@ -761,9 +768,18 @@ __device__ void warp_cf_run(BRun& r, const BCluster& c, const BTable* tabs, T* V
     int next_check = 32, hits = 0;
     const double sgn = create ? -1.0 : 1.0;
     double2 prev0 = make_double2(0.0, 0.0), prev1 = make_double2(0.0, 0.0);  // check frequencies lane, lane + 32
+    CfForward st0, st1;
+    int checked = 0;
+    warp_diag<T>(tu, td, c.hp, D);
+    const T* val;
+    if constexpr (sizeof(T) == 8)
+      val = c.hp.val;
+    else
+      val = c.hp.valf;
+    __syncwarp();
     for (int k = 0; k < r.mmax; ++k) {
       double sxw, sww, sxx;
-      warp_hx<T>(tu, td, c.hp, X, P, (T)bprev, sxw, sww, sxx);
+      warp_hx<T>(tu, td, D, val, X, P, (T)bprev, sxw, sww, sxx);
       const double alpha = sxx > 0.0 ? sxw / sxx : 0.0;
       const double b2 = sxx > 0.0 ? sww - sxw * sxw / sxx : 0.0;
       const double bn = b2 > 0.0 ? sqrt(b2) : 0.0;
@@ -783,15 +799,16 @@ __device__ void warp_cf_run(BRun& r, const BCluster& c, const BTable* tabs, T* V
       if (steps == next_check) {
         double mx = 0.0;
         if (lane < nzs) {
-          const double2 gv = b_cf_eval(r.alpha, r.beta, steps, s2, z[lane * zstride], c.E0, sgn);
+          const double2 gv = cf_advance(st0, r.alpha, r.beta, checked, steps, s2, z[lane * zstride], c.E0, sgn);
           mx = fmax(mx, hypot(gv.x - prev0.x, gv.y - prev0.y));
           prev0 = gv;
         }
         if (lane + 32 < nzs) {
-          const double2 gv = b_cf_eval(r.alpha, r.beta, steps, s2, z[(lane + 32) * zstride], c.E0, sgn);
+          const double2 gv = cf_advance(st1, r.alpha, r.beta, checked, steps, s2, z[(lane + 32) * zstride], c.E0, sgn);
           mx = fmax(mx, hypot(gv.x - prev1.x, gv.y - prev1.y));
           prev1 = gv;
         }
+        checked = steps;
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         hits = mx < tol ? hits + 1 : 0;
         if (hits >= 2) break;
@@ -839,7 +856,10 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
       g.sUf[i] = c.hp.Uf[i];
       g.sUd[i] = c.hp.U[i];
     }
-    for (int i = threadIdx.x; i < 4 * 64; i += blockDim.x) g.prev[i >> 6][i & 63] = make_double2(0.0, 0.0);
+    for (int i = threadIdx.x; i < 4 * 64; i += blockDim.x) {
+      g.prev[i >> 6][i & 63] = make_double2(0.0, 0.0);
+      g.st[i >> 6][i & 63] = CfForward{};
+    }
     const BTable tu = tabs[r0.tu], td = tabs[r0.td], src = tabs[r0.src];
     const BTable dst = r0.spin == 0 ? tu : td;
     const int64_t dd = td.dim, nel = r0.d;
@@ -904,7 +924,7 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
       __syncthreads();
     }
     bool active[4];
-    int steps[4], next_check[4], hits[4];
+    int steps[4], next_check[4], hits[4], checked[4];
     double bprev[4];
     T f[4];
 #pragma unroll
@@ -914,6 +934,7 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
       steps[q] = 0;
       next_check[q] = 32;
       hits[q] = 0;
+      checked[q] = 0;
       bprev[q] = 0.0;
     }
     for (int64_t idx = threadIdx.x; idx < nel; idx += blockDim.x) {
@@ -975,13 +996,16 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
         const BRun& rq = R[rid[q]];
         double mx = 0.0;
         for (int qq = threadIdx.x; qq < nzs; qq += blockDim.x) {
-          const double2 gv = b_cf_eval(rq.alpha, rq.beta, steps[q], s2[q], z[qq * zstride], c.E0, sgn);
+          CfForward st = g.st[q][qq];
+          const double2 gv = cf_advance(st, rq.alpha, rq.beta, checked[q], steps[q], s2[q], z[qq * zstride], c.E0, sgn);
+          g.st[q][qq] = st;
           mx = fmax(mx, hypot(gv.x - g.prev[q][qq].x, gv.y - g.prev[q][qq].y));
           g.prev[q][qq] = gv;
         }
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
         if ((threadIdx.x & 31) == 0) atomicMax((unsigned long long*)&g.maxdiff, __double_as_longlong(mx));
         __syncthreads();
+        checked[q] = steps[q];
         hits[q] = g.maxdiff < tol ? hits[q] + 1 : 0;
         if (hits[q] >= 2) active[q] = false;
         next_check[q] = steps[q] + max(32, steps[q] / 8);
@@ -995,18 +1019,31 @@ __global__ void __launch_bounds__(512) k_batch_cf(BRun* __restrict__ R, const in
       }
     __syncthreads();
   }
-  // warp phase
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T* W0 = reinterpret_cast<T*>(ws) + (int64_t)warp * 2 * w.wmax;
+  // warp phase.  FP64 sectors are bound by the FP64 pipe of their SM, so the largest runs must not
+  // share one: without block-level groups in front, warp w of block b starts with run w gridDim + b
+  // of the size order (blocks are dealt to the SMs in turn), then takes from the queue.  Taking every
+  // run from the queue put neighbours in the order on one SM: 64 clusters of at most 7 orbitals took
+  // 185 ms, 146 ms this way (with the hops four at a time, the diagonal once per run and incremental
+  // checks).
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  T* W0 = reinterpret_cast<T*>(ws) + (int64_t)warp * 3 * w.wmax;
   T* W1 = W0 + w.wmax;
+  T* W2 = W1 + w.wmax;
+  const int dealt = n_groups == 0 ? (int)gridDim.x * nwarp : 0;
+  bool deal = dealt > 0;
   while (true) {
     int t = 0;
-    if (lane == 0) t = atomicAdd(queue + 1, 1);
-    t = __shfl_sync(0xffffffffu, t, 0);
+    if (deal) {
+      t = warp * (int)gridDim.x + (int)blockIdx.x;
+      deal = false;
+    } else {
+      if (lane == 0) t = dealt + atomicAdd(queue + 1, 1);
+      t = __shfl_sync(0xffffffffu, t, 0);
+    }
     const int item = n_block + t;
     if (item >= n) return;
     BRun& r = R[order[item]];
-    warp_cf_run<T>(r, C[r.cluster], tabs, W0, W1, z, nz, tol);
+    warp_cf_run<T>(r, C[r.cluster], tabs, W0, W1, W2, z, nz, tol);
   }
 }
 
@@ -1178,7 +1215,7 @@ size_t batch_device_bytes(const ed_cluster_desc* descs, int n, int precision, in
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(n + nruns, (int64_t)sms * 4));
   const int64_t wmax = std::min<int64_t>(maxd, kWarpRunMax);
   const size_t stride = std::max<size_t>(std::max<size_t>(((3 * maxd * es + 255) / 256) * 256 + 4 * maxd * 8,
-                                                          (size_t)16 * 2 * wmax * es),
+                                                          (size_t)16 * 3 * wmax * es),
                                          (size_t)8 * maxd * es) + 256;
   return bytes + (size_t)blocks * stride + (size_t(1) << 20);
 }
@@ -1388,12 +1425,12 @@ void batch_solve(const ed_cluster_desc* descs, int n, int precision, const doubl
   for (int c = 0; c < n; ++c) maxd = std::max(maxd, C[c].d);
   for (int r = 0; r < nruns; ++r) maxd = std::max(maxd, R[r].d);
   const size_t es = precision == ED_FP64 ? 8 : 4;
-  // per block: 3 + 4 vectors of the largest sector, or 2 vectors per warp (at most 16) of the
+  // per block: 3 + 4 vectors of the largest sector, or 3 vectors per warp (at most 16) of the
   // largest warp-level run, whichever is more
   const int64_t wmax = std::min<int64_t>(maxd, kWarpRunMax);
   // (or two sets of four interleaved vectors of a group of block-level continued fractions)
   const size_t stride = std::max<size_t>(std::max<size_t>(((3 * maxd * es + 255) / 256) * 256 + 4 * maxd * 8,
-                                                          (size_t)16 * 2 * wmax * es),
+                                                          (size_t)16 * 3 * wmax * es),
                                          (size_t)8 * maxd * es) + 256;
   int dev = 0, sms = 0;
   ED_CUDA(cudaGetDevice(&dev));
@@ -1406,11 +1443,16 @@ void batch_solve(const ed_cluster_desc* descs, int n, int precision, const doubl
   int nbucket = 0;
   while ((1 << nbucket) < n) ++nbucket;
   const auto key = std::make_tuple(Lmax, dbucket, nbucket, precision);
-  std::pair<int, int> cfg{256, 0};
-  bool tuned = fixed_threads > 0;
-  if (tuned) {
+  // Sectors that all take the warp-level fractions use 128 threads: the block-level part is then
+  // only the ground states of small sectors, mostly the tridiagonal checks, which four warps serve
+  // as well as sixteen.  A width picked by timing the ground states alone could double the time of
+  // the fractions (64 clusters of at most 7 orbitals: 185 ms with 128 threads, 292 ms otherwise), and
+  // made the order of the sums hang on a timing.
+  std::pair<int, int> cfg{128, 0};
+  bool tuned = fixed_threads > 0 || maxd <= kWarpRunMax;
+  if (fixed_threads > 0) {
     cfg = {fixed_threads, fixed_mode};
-  } else {
+  } else if (!tuned) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
     tuned = it != g_tune.end();
