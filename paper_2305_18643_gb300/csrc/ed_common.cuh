@@ -201,6 +201,7 @@ struct SectorView {
   const double* e_dn;
   const float* e_up32;
   const float* e_dn32;
+  int zmax_up;              // most hops of an up-spin state
   int64_t two_pass_min_bytes;  // vectors of at least this many bytes take the two-pass H.psi
 };
 

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kStaticThreads) k_hpsi_dots_static(SectorView 
     const int64_t idx = ((int64_t)blockIdx.x * kStaticPerThread + k) * kStaticThreads + threadIdx.x;
     if (idx >= dim) break;
     const int64_t u = idx / sv.d_dn, d = idx - u * sv.d_dn;
-    const T acc = hpsi_element<T>(sv, sval, sU, hp.umask, X, u, d);
+    const T acc = hpsi_element<T>(sv, sval, sU, hp, X, u, d);
     Y[u * sv.ld + d] = acc;
     const double xv = (double)X[u * sv.ld + d], yv = (double)acc;
     sxy += xv * yv;

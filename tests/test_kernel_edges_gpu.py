@@ -105,3 +105,39 @@ def test_continued_fraction_grid_edges(nz):
         assert np.abs(cl.green(om, 0.05) - ref).max() <= 1e-8
     G = ed.ed_batch_solve([c], omega=om, eta=0.05, seed=5)[4][0]
     assert np.abs(G[0] - ref).max() <= 1e-8 and np.abs(G[1] - ref).max() <= 1e-8
+
+
+# One-pass H.psi: flat index below 192 columns, tiles of 4, 2 and 1 rows with ragged last tiles and
+# column chunks, rows too long for shared memory; padded rows keep their padding.  FP64 within 1e-12
+# and FP32 within 2e-5 of max|y| (the bounds of the parity tests).
+@pytest.mark.parametrize("L,n_up,n_dn", [(2, 1, 1), (20, 1, 2), (21, 1, 2), (10, 5, 5), (12, 1, 6), (12, 6, 5), (16, 3, 8),
+                                         (18, 1, 8), (24, 1, 6)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("pad", [0, 3])
+def test_one_pass_hpsi_forms(L, n_up, n_dn, dtype, pad):
+    rng = np.random.default_rng(L + n_up)
+    c = W.random_cluster(rng, L, 0, n_up, n_dn, U=4.0 if pad else None, dense_t=L <= 12)
+    op = O.sector_hamiltonian(_model(c), n_up, n_dn)
+    with ed.Cluster(c) as cl:
+        du, dd = ed.ed_sector_dims(cl.h, n_up, n_dn)
+        x = rng.standard_normal((du, dd))
+        xd = torch.zeros((du, dd + pad), dtype=dtype, device="cuda")
+        xd[:, :dd] = torch.tensor(x, device="cuda")
+        y = torch.full((du, dd + pad), 7.0, dtype=dtype, device="cuda")
+        ed.ed_hpsi(cl.h, n_up, n_dn, ed.ED_FP64 if dtype == torch.float64 else ed.ED_FP32, xd.data_ptr(), y.data_ptr(),
+                   dd + pad, torch.cuda.current_stream().cuda_stream)
+        got = y.cpu().double().numpy()
+    ref = O.apply_h(op, xd[:, :dd].cpu().double().numpy()).reshape(du, dd)
+    tol = 1e-12 if dtype == torch.float64 else 2e-5
+    assert np.abs(got[:, :dd] - ref).max() <= tol * np.abs(ref).max()
+    assert np.all(got[:, dd:] == 7.0)
+
+
+# The fused step of the one-pass forms through whole solves (E0 within 1e-10 of the oracle).
+@pytest.mark.parametrize("L,n_up,n_dn", [(6, 1, 3), (10, 5, 4), (12, 2, 6)])
+@pytest.mark.parametrize("precision", [ed.ED_FP64, ed.ED_FP32])
+def test_one_pass_lanczos_forms(L, n_up, n_dn, precision):
+    c = W.random_cluster(np.random.default_rng(L), L, 0, n_up, n_dn)
+    E = O.ground_state(O.sector_hamiltonian(_model(c), n_up, n_dn))[0]
+    with ed.Cluster(c, seed=5, precision=precision) as cl:
+        assert abs(cl.ground_state()[1] - np.min(E)) <= 1e-10 * abs(np.min(E))
