@@ -274,6 +274,15 @@ void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, c
 int lanczos_blocks(const SectorView& sv);   // partial-sum slots per run of the fused step
 int two_pass_blocks(const SectorView& sv, int dtype);
 
+// small.cu: many Lanczos levels of small sectors in one launch, a thread-block cluster per run.
+struct SmallStore {  // where the vectors v_{n0 + 1}, v_{n0 + 2}, ... are kept too
+  void* p[16];
+  int count;
+};
+int small_cluster_size(const SectorView& sv, int dtype, int runs, double hops);
+void launch_small_levels(const SectorView& sv, const HopParams& hp, int dtype, void* V, void* VP, int64_t vstride, int runs,
+                         int n0, int n1, const LanczosScalars& ls, int nb, const SmallStore& store, cudaStream_t s);
+
 // lanczos.cu
 // omega (contiguous) += coef[n + 1] v_{n+1}; its type is omega_dtype (< 0: the vectors' dtype).
 void launch_lanczos_next(int dtype, void* W, const void* X, int64_t d_up, int64_t d_dn, int64_t ld,

@@ -303,10 +303,19 @@ static bool cf_part(ed_cluster& c, int spin, bool electron, int dtype, const Dev
     char* V[2] = {V0.p, V1.p};
     int cur = 0;
     int next_check = 32;
+    // small sectors: all levels up to the next check in one launch
+    const double hops = (double)c.tables(nu_t).nnz / c.tables(nu_t).dim + (double)c.tables(nd_t).nnz / c.tables(nd_t).dim;
+    const int nb = small_cluster_size(sv, dtype, rc, hops);
     for (int n = 0; n < M; ++n) {
-      launch_lanczos_step(sv, c.hp, dtype, V[cur], V[cur ^ 1], vstride, rc, n, ls, nblk, s);
-      launch_lanczos_next(dtype, V[cur ^ 1], V[cur], du, dd, ld, vstride, rc, n, ls, nullptr, nullptr, s);
-      cur ^= 1;
+      if (nb) {
+        const int n1 = std::min(next_check, M);
+        launch_small_levels(sv, c.hp, dtype, V[0], V[1], vstride, rc, n, n1, ls, nb, SmallStore{}, s);
+        n = n1 - 1;
+      } else {
+        launch_lanczos_step(sv, c.hp, dtype, V[cur], V[cur ^ 1], vstride, rc, n, ls, nblk, s);
+        launch_lanczos_next(dtype, V[cur ^ 1], V[cur], du, dd, ld, vstride, rc, n, ls, nullptr, nullptr, s);
+        cur ^= 1;
+      }
       if (n + 1 == next_check || n + 1 == M) {
         ED_CUDA(cudaMemsetAsync(nact.p, 0, sizeof(int), s));
         {

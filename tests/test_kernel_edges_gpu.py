@@ -141,3 +141,17 @@ def test_one_pass_lanczos_forms(L, n_up, n_dn, precision):
     E = O.ground_state(O.sector_hamiltonian(_model(c), n_up, n_dn))[0]
     with ed.Cluster(c, seed=5, precision=precision) as cl:
         assert abs(cl.ground_state()[1] - np.min(E)) <= 1e-10 * abs(np.min(E))
+
+
+# Levels of small sectors in clusters of 1 to 8 blocks: sectors of a few states (most blocks own
+# nothing) up to 1,225, both precisions, both spins.  FP64 within 1e-8 of the exact Lehmann sum, FP32
+# vectors within 2e-4 (the bounds of the parity tests on the real axis at eta = 0.05).
+@pytest.mark.parametrize("L,n_up,n_dn", [(2, 1, 1), (3, 1, 2), (5, 2, 3), (7, 3, 4)])
+@pytest.mark.parametrize("precision,tol", [(ed.ED_FP64, 1e-8), (ed.ED_FP32, 2e-4)])
+def test_small_sector_levels(L, n_up, n_dn, precision, tol):
+    c = W.random_cluster(np.random.default_rng(7 * L), L, 0, n_up, n_dn)
+    om = np.linspace(-8.0, 8.0, 101)
+    with ed.Cluster(c, seed=5, precision=precision) as cl:
+        for spin in (0, 1):
+            ref = O.green_exact(_model(c), n_up, n_dn, om + 0.05j, spin=spin)[0]
+            assert np.abs(cl.green(om, 0.05, spin=spin) - ref).max() <= tol
