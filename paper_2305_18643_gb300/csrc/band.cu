@@ -155,8 +155,15 @@ struct GPartOf<double> {
 // it over the tile, GR 16-byte groups per lane (rows padded by 16 bytes: conflict-free 16-byte
 // shared loads).  Products are summed per pair over kGramFlush tiles (FP32: packed FMAs), then
 // added with compensation; lanes, chunks and blocks are added in a fixed order, the chunks by
-// the last CTA of each X block (a ticket), so the result is deterministic.
+// the last CTA of each X block (a ticket), so the result is deterministic.  With fewer than 16 pair
+// tiles (blocks narrower than 13 vectors) SPLIT warps share a tile, each taking every SPLIT-th group of
+// elements: FP64 products are bound by the FP64 pipes of the four SM sub-partitions, and one warp per
+// CTA kept one of them busy (4 vectors against 4, 811,008 elements, FP64: 68 us in place of 154 us
+// on average over 1 to 25 blocks).
 constexpr int kGramFlush = 4;
+__host__ __device__ constexpr int gram_split(int tiles, int gr) {
+  return tiles <= 4 ? (gr < 4 ? gr : 4) : tiles <= 8 ? (gr < 2 ? gr : 2) : 1;
+}
 template <typename T, int GR>
 __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T* __restrict__ X0, const T* __restrict__ X1,
                                                          int64_t xbstride, int px, const T* __restrict__ Y, int py,
@@ -180,7 +187,8 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T* __restrict__ 
   const int ntile = e_begin < e_end ? (int)((e_end - e_begin + E - 1) / E) : 0;  // the last may be partial
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int TI = (px + 3) / 4, TJ = (py + 3) / 4;
-  const int q0 = blockIdx.z * kGramTilesPerCta + warp;
+  const int split = gram_split(TI * TJ, GR), sub = warp % split;
+  const int q0 = blockIdx.z * kGramTilesPerCta + warp / split;
   const bool h0 = q0 < TI * TJ;
   const int ti0 = h0 ? q0 / TJ : 0, tj0 = h0 ? q0 % TJ : 0;
   auto stage = [&](int t) {
@@ -215,6 +223,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T* __restrict__ 
     if (h0) {
 #pragma unroll
       for (int g = 0; g < GR; ++g) {
+        if (g % split != sub) continue;
         const T* bg = b + g * 32 * VN;
         V xv[4], yv[4];
 #pragma unroll
@@ -236,7 +245,7 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T* __restrict__ 
   }
   cp_async_wait<0>();
   const int npair = px * py;
-  double* Pc = P + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * npair;
+  double* Pc = P + (((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * split + sub) * npair;
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     double v0 = acc0[k].get();
@@ -255,11 +264,14 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram(const T* __restrict__ 
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const double* Pb = P + (int64_t)blockIdx.y * gridDim.x * npair;
-  for (int q = threadIdx.x; q < npair; q += blockDim.x) {
+  // a warp per pair: lanes over the chunks, then a fixed tree (one thread per pair would add hundreds
+  // of partials one after the other)
+  const double* Pb = P + (int64_t)blockIdx.y * gridDim.x * split * npair;
+  for (int q = warp; q < npair; q += kGramTilesPerCta) {
     double v = 0.0;
-    for (unsigned c = 0; c < gridDim.x; ++c) v += __ldcg(Pb + (int64_t)c * npair + q);
-    G[(int64_t)blockIdx.y * npair + q] = v;
+    for (int c = lane; c < (int)gridDim.x * split; c += 32) v += __ldcg(Pb + (int64_t)c * npair + q);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) G[(int64_t)blockIdx.y * npair + q] = v;
   }
   if (threadIdx.x == 0) ticket[blockIdx.y] = 0u;
 }
@@ -332,27 +344,32 @@ __global__ void __launch_bounds__(kGT2) k_block_axpy(T* __restrict__ Y, int py, 
 // ---- small dense work of one block step (one thread block) ---------------------------------
 // SVQB of a block with Gram G: Cout = U l^{-1/2} (new basis = W Cout), Bout = l^{1/2} U^T
 // (W = new basis * Bout); directions with l <= thr are dropped (zero columns / rows).  Writes
-// the number of kept directions to *rank.  Parallel two-sided Jacobi on one warp: every round
-// applies m/2 disjoint rotations at once (round-robin pairing of the m = p rounded up to even
-// indices; an index >= p is a dummy), A <- J^T A J with J block-diagonal, so a sweep is m - 1
-// rounds.  Sweeps stop when the off-diagonal norm is below 1e-26 of the total.
-__global__ void __launch_bounds__(32) k_svqb(const double* __restrict__ G, int p, double thr,
-                                             double* __restrict__ Cout, double* __restrict__ Bout,
-                                             int* __restrict__ rank) {
+// the number of kept directions to *rank.  Parallel two-sided Jacobi: every round applies m/2
+// disjoint rotations at once (round-robin pairing of the m = p rounded up to even indices; an index
+// >= p is a dummy), A <- J^T A J with J block-diagonal, so a sweep is m - 1 rounds.  Sweeps stop when
+// the off-diagonal norm is below 1e-26 of the total.  The rounds are a chain of FP64 latencies: the
+// tangent of an angle is an FP32 quotient (an angle off by 1e-7 leaves 1e-7 of the entry it removes),
+// its cosine FP64, and four warps, one per SM sub-partition, share the updates.  p = 14: 357 us with one
+// warp and FP64 quotients, 127 us now.
+constexpr int kSvqbThreads = 128;
+__global__ void __launch_bounds__(kSvqbThreads) k_svqb(const double* __restrict__ G, int p, double thr,
+                                                       double* __restrict__ Cout, double* __restrict__ Bout,
+                                                       int* __restrict__ rank) {
   __shared__ double a[kBP][kBP + 1], v[kBP][kBP + 1];
   __shared__ double cs[kBP / 2], sn[kBP / 2];
   __shared__ int pr[kBP / 2], pq[kBP / 2];
-  const int lane = threadIdx.x;
-  for (int t = lane; t < p * p; t += 32) {
+  __shared__ double s_off[kSvqbThreads / 32], s_tot[kSvqbThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int t = tid; t < p * p; t += kSvqbThreads) {
     const int i = t / p, j = t - i * p;
     a[i][j] = 0.5 * (G[i * p + j] + G[j * p + i]);
     v[i][j] = i == j ? 1.0 : 0.0;
   }
-  __syncwarp();
+  __syncthreads();
   const int m = p + (p & 1), half = m / 2;
   for (int sweep = 0; sweep < 40; ++sweep) {
     double off = 0.0, tot = 0.0;
-    for (int t = lane; t < p * p; t += 32) {
+    for (int t = tid; t < p * p; t += kSvqbThreads) {
       const int i = t / p, j = t - i * p;
       tot += a[i][j] * a[i][j];
       if (i != j) off += a[i][j] * a[i][j];
@@ -361,10 +378,18 @@ __global__ void __launch_bounds__(32) k_svqb(const double* __restrict__ G, int p
       off += __shfl_xor_sync(0xffffffffu, off, o);
       tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
+    if (lane == 0) {
+      s_off[warp] = off;
+      s_tot[warp] = tot;
+    }
+    __syncthreads();
+    off = s_off[0] + s_off[1] + s_off[2] + s_off[3];
+    tot = s_tot[0] + s_tot[1] + s_tot[2] + s_tot[3];
+    __syncthreads();
     if (!(off > 1e-26 * tot)) break;
     for (int round = 0; round < m - 1; ++round) {
-      if (lane < half) {  // pair lane: positions lane and m - 1 - lane of the round-robin circle
-        const int pa = lane, pb = m - 1 - lane;
+      if (tid < half) {  // pair tid: positions tid and m - 1 - tid of the round-robin circle
+        const int pa = tid, pb = m - 1 - tid;
         int r = pa == 0 ? 0 : 1 + (pa - 1 + round) % (m - 1);
         int q = pb == 0 ? 0 : 1 + (pb - 1 + round) % (m - 1);
         if (r > q) {
@@ -374,22 +399,22 @@ __global__ void __launch_bounds__(32) k_svqb(const double* __restrict__ G, int p
         }
         double c = 1.0, s = 0.0;
         if (q < p) {
-          const double arq = a[r][q];
-          if (fabs(arq) >= 1e-300) {
-            const double theta = (a[q][q] - a[r][r]) / (2.0 * arq);
-            const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
+          const float arq = (float)a[r][q];
+          if (arq != 0.f) {
+            const float theta = (float)(a[q][q] - a[r][r]) / (2.f * arq);
+            const double t = (double)((theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f))));
+            c = rsqrt(fma(t, t, 1.0));
             s = t * c;
           }
         }
-        pr[lane] = r;
-        pq[lane] = q < p ? q : r;  // a dummy pair becomes (r, r) and is skipped below
-        cs[lane] = c;
-        sn[lane] = s;
+        pr[tid] = r;
+        pq[tid] = q < p ? q : r;  // a dummy pair becomes (r, r) and is skipped below
+        cs[tid] = c;
+        sn[tid] = s;
       }
-      __syncwarp();
+      __syncthreads();
       // columns: A <- A J, V <- V J
-      for (int t = lane; t < half * p; t += 32) {
+      for (int t = tid; t < half * p; t += kSvqbThreads) {
         const int i = t / p, k = t - i * p, r = pr[i], q = pq[i];
         if (r == q) continue;
         const double c = cs[i], s = sn[i];
@@ -400,9 +425,9 @@ __global__ void __launch_bounds__(32) k_svqb(const double* __restrict__ G, int p
         v[k][r] = c * vkr - s * vkq;
         v[k][q] = s * vkr + c * vkq;
       }
-      __syncwarp();
+      __syncthreads();
       // rows: A <- J^T A
-      for (int t = lane; t < half * p; t += 32) {
+      for (int t = tid; t < half * p; t += kSvqbThreads) {
         const int i = t / p, k = t - i * p, r = pr[i], q = pq[i];
         if (r == q) continue;
         const double c = cs[i], s = sn[i];
@@ -410,20 +435,19 @@ __global__ void __launch_bounds__(32) k_svqb(const double* __restrict__ G, int p
         a[r][k] = c * ark - s * aqk;
         a[q][k] = s * ark + c * aqk;
       }
-      __syncwarp();
+      __syncthreads();
     }
   }
-  __syncwarp();
   int r = 0;
   for (int k = 0; k < p; ++k) r += a[k][k] > thr;
-  for (int t = lane; t < p * p; t += 32) {
+  for (int t = tid; t < p * p; t += kSvqbThreads) {
     const int i = t / p, k = t - i * p;
     const double l = a[k][k];
     const bool keep = l > thr;
     Cout[i * p + k] = keep ? v[i][k] / sqrt(l) : 0.0;
     Bout[k * p + i] = keep ? v[i][k] * sqrt(l) : 0.0;
   }
-  if (lane == 0) *rank = r;
+  if (tid == 0) *rank = r;
 }
 
 // out = a * b (p x p), optionally transposing b: used to chain the two SVQB factors and to form
@@ -467,102 +491,112 @@ struct BandCoeffs {
   double E0, sgn;    // sgn = +1 electron (s = z + E0, M = s - A), -1 hole (s = z - E0, M = s + A)
 };
 
-// One thread block per frequency: complex p x p matrices in shared memory.
-__global__ void __launch_bounds__(256) k_band_cf(BandCoeffs bc, const double2* __restrict__ z, int nz, int zstride,
-                                                 double2* __restrict__ out /* [nz][p][p] */, double2* __restrict__ prev,
-                                                 double* __restrict__ maxdiff) {
-  __shared__ double2 M[kBP][kBP + 1];
-  __shared__ double2 Y[kBP][2 * kBP + 1];
-  __shared__ double2 fcol[kBP];
-  const int zi = blockIdx.x;
-  if (zi * zstride >= nz) return;
-  const double2 zz = z[zi * zstride];
-  const int p = bc.p;
+// A group of M lanes per frequency (M = p rounded up to a power of two, 32 / M frequencies per warp), lane
+// b holding column b of the complex symmetric matrix and of the right-hand side in registers, so no
+// barriers and no idle lanes.  With M_{j+1} = L D L^T (no pivoting), B^T M_{j+1}^{-1} B = Z^T D^{-1} Z for
+// Z = L^{-1} B: forward elimination alone; row k of Z contributes when it is final.  The rows rotate
+// through the registers as they are eliminated, so every index is static.
+// FP64-bound.  p = 4, 1,000 frequencies, up to 25 levels: 969 us a launch with a thread block and
+// shared matrices per frequency, 164 us now; p = 14: 1,460 us and 595 us.
+constexpr int kBandCfThreads = 64;
+template <int M>
+__global__ void __launch_bounds__(kBandCfThreads) k_band_cf(BandCoeffs bc, const double2* __restrict__ z, int nz, int zstride,
+                                                            double2* __restrict__ out /* [nz][p][p] */,
+                                                            double2* __restrict__ prev, double* __restrict__ maxdiff) {
+  const int p = bc.p, pp = p * p;
+  const int lane = threadIdx.x & 31, b = lane & (M - 1);
+  const int zi = (blockIdx.x * kBandCfThreads + threadIdx.x) / M;
+  const bool mine = (int64_t)zi * zstride < nz;
+  const int bb = b < p ? b : 0;  // lanes past p repeat column 0 and write nothing
+  const double2 zz = mine ? z[(int64_t)zi * zstride] : make_double2(0.0, 1.0);
   const double2 s = make_double2(zz.x + bc.sgn * bc.E0, zz.y);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  auto init_M = [&](int j) {
-    for (int t = tid; t < p * p; t += nt) {
-      const int a = t / p, b = t - a * p;
-      double v = -bc.sgn * bc.A[((int64_t)j * p + a) * p + b];
-      M[a][b] = make_double2((a == b ? s.x : 0.0) + v, a == b ? s.y : 0.0);
+  double2 c[M], r[M], t[M];
+  // t <- column b of R^T C^{-1} R for the matrix with columns c (R: p x p, row-major)
+  auto project = [&](const double* __restrict__ R) {
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      r[i] = make_double2(i < p ? R[i * p + bb] : 0.0, 0.0);
+      t[i] = make_double2(0.0, 0.0);
+    }
+    for (int k = 0; k < p; ++k) {
+      // pivot row k is register 0: d = c[0] of lane k, z_k[b] = r[0]
+      const double2 d = make_double2(__shfl_sync(0xffffffffu, c[0].x, k, M), __shfl_sync(0xffffffffu, c[0].y, k, M));
+      const double den = 1.0 / (d.x * d.x + d.y * d.y);
+      const double2 id = make_double2(d.x * den, -d.y * den);
+      const double2 w = make_double2(r[0].x * id.x - r[0].y * id.y, r[0].x * id.y + r[0].y * id.x);    // z_k[b] / d
+      const double2 cw = make_double2(c[0].x * id.x - c[0].y * id.y, c[0].x * id.y + c[0].y * id.x);   // row k of c / d
+#pragma unroll
+      for (int a = 0; a < M; ++a) {
+        if (a < p) {
+          const double zr = __shfl_sync(0xffffffffu, r[0].x, a, M), zim = __shfl_sync(0xffffffffu, r[0].y, a, M);
+          t[a] = make_double2(fma(zr, w.x, fma(-zim, w.y, t[a].x)), fma(zr, w.y, fma(zim, w.x, t[a].y)));
+        }
+      }
+#pragma unroll
+      for (int i = 1; i < M; ++i) {
+        if (i < p - k) {
+          const double fr = __shfl_sync(0xffffffffu, c[i].x, k, M), fi = __shfl_sync(0xffffffffu, c[i].y, k, M);
+          c[i - 1] = make_double2(fma(-fr, cw.x, fma(fi, cw.y, c[i].x)), fma(-fr, cw.y, fma(-fi, cw.x, c[i].y)));
+          r[i - 1] = make_double2(fma(-fr, w.x, fma(fi, w.y, r[i].x)), fma(-fr, w.y, fma(-fi, w.x, r[i].y)));
+        }
+      }
     }
   };
-  // Solve M Y = rhs (rhs p x m, real) in place: augmented [M | rhs] in Y, no pivoting.
-  auto solve = [&](const double* rhs, int m, bool rhs_t) {
-    for (int t = tid; t < p * (p + m); t += nt) {
-      const int a = t / (p + m), b = t - a * (p + m);
-      if (b < p)
-        Y[a][b] = M[a][b];
-      else {
-        const double r = rhs_t ? rhs[(b - p) * p + a] : rhs[a * p + (b - p)];
-        Y[a][b] = make_double2(r, 0.0);
+  for (int j = bc.k - 1; j >= 0; --j) {
+    // M_j = s -/+ A_j - B_j^T M_{j+1}^{-1} B_j
+    if (j < bc.k - 1) project(bc.B + (int64_t)j * pp);
+    const double* A = bc.A + (int64_t)j * pp;
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+      if (a < p) {
+        const double v = -bc.sgn * A[a * p + bb];
+        const double2 q = j < bc.k - 1 ? t[a] : make_double2(0.0, 0.0);
+        c[a] = make_double2((a == bb ? s.x : 0.0) + v - q.x, (a == bb ? s.y : 0.0) - q.y);
       }
     }
-    __syncthreads();
-    for (int c = 0; c < p; ++c) {
-      const double2 piv = Y[c][c];
-      const double den = piv.x * piv.x + piv.y * piv.y;
-      const double2 ip = make_double2(piv.x / den, -piv.y / den);
-      __syncthreads();
-      for (int t = tid; t < p + m; t += nt) {  // scale pivot row
-        const double2 v = Y[c][t];
-        if (t >= c) Y[c][t] = make_double2(v.x * ip.x - v.y * ip.y, v.x * ip.y + v.y * ip.x);
-      }
-      for (int t = tid; t < p; t += nt) fcol[t] = Y[t][c];
-      __syncthreads();
-      for (int t = tid; t < p * (p + m); t += nt) {
-        const int a = t / (p + m), b = t - a * (p + m);
-        if (a == c || b < c) continue;
-        const double2 f = fcol[a], v = Y[c][b];
-        Y[a][b].x -= f.x * v.x - f.y * v.y;
-        Y[a][b].y -= f.x * v.y + f.y * v.x;
-      }
-      __syncthreads();
-    }
-  };
-  init_M(bc.k - 1);
-  __syncthreads();
-  for (int j = bc.k - 2; j >= 0; --j) {
-    // Y = M_{j+1}^{-1} B_j  (B_j: p x p, row index = new-basis direction)
-    solve(bc.B + (int64_t)j * p * p, p, false);
-    // M_j = s -/+ A_j - B_j^T Y
-    for (int t = tid; t < p * p; t += nt) {
-      const int a = t / p, b = t - a * p;
-      double2 acc = make_double2(0.0, 0.0);
-      for (int k2 = 0; k2 < p; ++k2) {
-        const double bk = bc.B[((int64_t)j * p + k2) * p + a];
-        acc.x += bk * Y[k2][p + b].x;
-        acc.y += bk * Y[k2][p + b].y;
-      }
-      const double v = -bc.sgn * bc.A[((int64_t)j * p + a) * p + b];
-      M[a][b] = make_double2((a == b ? s.x : 0.0) + v - acc.x, (a == b ? s.y : 0.0) - acc.y);
-    }
-    __syncthreads();
   }
-  // G = R0^T M_1^{-1} R0
-  solve(bc.R0, p, false);
+  project(bc.R0);  // G = R0^T M_1^{-1} R0
   double local = 0.0;
-  for (int t = tid; t < p * p; t += nt) {
-    const int a = t / p, b = t - a * p;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k2 = 0; k2 < p; ++k2) {
-      const double r = bc.R0[k2 * p + a];
-      acc.x += r * Y[k2][p + b].x;
-      acc.y += r * Y[k2][p + b].y;
-    }
-    const int64_t o = (int64_t)zi * p * p + t;
-    if (prev) {
-      const double2 q = prev[o];
-      local = fmax(local, hypot(acc.x - q.x, acc.y - q.y));
-      prev[o] = acc;
-    } else {
-      out[o] = acc;
+  if (mine && b < p) {
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+      if (a < p) {
+        const int64_t o = (int64_t)zi * pp + a * p + b;
+        if (prev) {
+          const double2 q = prev[o];
+          local = fmax(local, hypot(t[a].x - q.x, t[a].y - q.y));
+          prev[o] = t[a];
+        } else {
+          out[o] = t[a];
+        }
+      }
     }
   }
   if (maxdiff) {
     for (int off = 16; off > 0; off >>= 1) local = fmax(local, __shfl_down_sync(0xffffffffu, local, off));
-    if ((tid & 31) == 0) atomicMax((unsigned long long*)maxdiff, __double_as_longlong(local));
+    if (lane == 0) atomicMax((unsigned long long*)maxdiff, __double_as_longlong(local));
   }
+}
+
+// The block continued fraction on every zstride-th of nz frequencies.
+static void band_cf(const BandCoeffs& bc, const double2* z, int nz, int zstride, double2* out, double2* prev,
+                    double* maxdiff, cudaStream_t s) {
+  const int n = (nz + zstride - 1) / zstride;
+  ProfScope ps_(K_GF_EVAL, s, 0.0);
+  auto go = [&](auto m) {
+    constexpr int M = decltype(m)::value;
+    constexpr int per = kBandCfThreads / M;
+    k_band_cf<M><<<(n + per - 1) / per, kBandCfThreads, 0, s>>>(bc, z, nz, zstride, out, prev, maxdiff);
+  };
+  if (bc.p <= 2)
+    go(std::integral_constant<int, 2>());
+  else if (bc.p <= 4)
+    go(std::integral_constant<int, 4>());
+  else if (bc.p <= 8)
+    go(std::integral_constant<int, 8>());
+  else
+    go(std::integral_constant<int, 16>());  // wider blocks are refused by block_axpy
+  ED_CHECK_LAUNCH();
 }
 
 // ---- driver -----------------------------------------------------------------------------------
@@ -585,7 +619,8 @@ static void gram_launch(const T* X, const T* X1, int64_t xbstride, int nb, int p
   const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, sms / (nb * gz))));
   const int64_t chunk = (tiles + nchunk - 1) / nchunk * E;
   const int npair = px * py;
-  if (P.n < (size_t)nb * nchunk * npair) P.alloc((size_t)nb * nchunk * npair);
+  const size_t parts = (size_t)nb * nchunk * gram_split(ntiles_pair, GR) * npair;
+  if (P.n < parts) P.alloc(parts);
   if (tk.n < (size_t)nb) {
     tk.alloc((size_t)nb);
     ED_CUDA(cudaMemsetAsync(tk.p, 0, (size_t)nb * sizeof(unsigned), s));
@@ -739,11 +774,11 @@ static bool band_part(ed_cluster& c, int spin, bool electron, const DevBuf<doubl
     // two SVQB passes: W = X (B2 B1); the second writes the orthonormal block into dst
     int r = 0;
     gram<T>(Wb.p, nullptr, 0, 1, p, Wb.p, p, vstride, n, P, gtk, G.p, s, &tc);
-    { ProfScope ps_(K_BAND, s, 0.0); k_svqb<<<1, 32, 0, s>>>(G.p, p, eps_rel * eps_rel * scale2, Cm.p, Bm.p, rank.p); }
+    { ProfScope ps_(K_BAND, s, 0.0); k_svqb<<<1, kSvqbThreads, 0, s>>>(G.p, p, eps_rel * eps_rel * scale2, Cm.p, Bm.p, rank.p); }
     ED_CHECK_LAUNCH();
     block_axpy<T>(Wb.p, p, Wb.p, nullptr, 0, 1, p, Cm.p, vstride, n, 0, s);
     gram<T>(Wb.p, nullptr, 0, 1, p, Wb.p, p, vstride, n, P, gtk, G.p, s, &tc);
-    { ProfScope ps_(K_BAND, s, 0.0); k_svqb<<<1, 32, 0, s>>>(G.p, p, 0.25, C2.p, B2.p, rank.p); }
+    { ProfScope ps_(K_BAND, s, 0.0); k_svqb<<<1, kSvqbThreads, 0, s>>>(G.p, p, 0.25, C2.p, B2.p, rank.p); }
     ED_CHECK_LAUNCH();
     block_axpy<T>(dst, p, Wb.p, nullptr, 0, 1, p, C2.p, vstride, n, 0, s);
     { ProfScope ps_(K_BAND, s, 0.0); k_small_gemm<<<1, 256, 0, s>>>(B2.p, Bm.p, p, 0, Bfinal, 1.0); }
@@ -804,8 +839,7 @@ static bool band_part(ed_cluster& c, int spin, bool electron, const DevBuf<doubl
     if (k == next_check || j + 1 == kmax) {
       BandCoeffs bc{A.p, B.p, R0.p, k, p, c.gs.E0, sgn};
       ED_CUDA(cudaMemsetAsync(dmax.p, 0, sizeof(double), s));
-      { ProfScope ps_(K_GF_EVAL, s, 0.0); k_band_cf<<<nzc, 256, 0, s>>>(bc, zd.p, nz, zstride, nullptr, prev.p, dmax.p); }
-      ED_CHECK_LAUNCH();
+      band_cf(bc, zd.p, nz, zstride, nullptr, prev.p, dmax.p, s);
       ED_CUDA(cudaMemcpyAsync(hmax, dmax.p, sizeof(double), cudaMemcpyDeviceToHost, s));
       ED_CUDA(cudaStreamSynchronize(s));
       if (*hmax < opt.tol) {
@@ -820,8 +854,7 @@ static bool band_part(ed_cluster& c, int spin, bool electron, const DevBuf<doubl
     }
   }
   BandCoeffs bc{A.p, B.p, R0.p, k, p, c.gs.E0, sgn};
-  { ProfScope ps_(K_GF_EVAL, s, 0.0); k_band_cf<<<nz, 256, 0, s>>>(bc, zd.p, nz, 1, Gout, nullptr, nullptr); }
-  ED_CHECK_LAUNCH();
+  band_cf(bc, zd.p, nz, 1, Gout, nullptr, nullptr, s);
   ED_CUDA(cudaStreamSynchronize(s));
   *total += (int64_t)k * p;
   *maxd = std::max(*maxd, k * p);

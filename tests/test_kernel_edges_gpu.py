@@ -155,3 +155,29 @@ def test_small_sector_levels(L, n_up, n_dn, precision, tol):
         for spin in (0, 1):
             ref = O.green_exact(_model(c), n_up, n_dn, om + 0.05j, spin=spin)[0]
             assert np.abs(cl.green(om, 0.05, spin=spin) - ref).max() <= tol
+
+
+# Band Lanczos at every group width of the block continued fraction (2, 4, 8, 16 lanes) and every split of
+# the Gram's warps (1, 4, 9 and 16 pair tiles), against the exact Lehmann sum (FP64, 1e-8).
+@pytest.mark.parametrize("ns,nb,n_up,n_dn", [(1, 5, 3, 3), (2, 4, 3, 2), (3, 3, 3, 3), (5, 1, 2, 3), (8, 0, 2, 1), (9, 0, 1, 1),
+                                             (14, 0, 1, 1)])
+def test_band_widths(ns, nb, n_up, n_dn):
+    c = W.random_cluster(np.random.default_rng(ns), ns, nb, n_up, n_dn)
+    om = W.matsubara_grid(33)
+    ref = O.green_exact(_model(c), n_up, n_dn, 1j * om)[0]
+    with ed.Cluster(c, seed=5, gf_method=ed.ED_GF_BAND) as cl:
+        assert np.abs(cl.green(om, 0.0, axis=ed.ED_AXIS_MATSUBARA) - ref).max() <= 1e-8
+
+
+# CUDA-core Gram with shared pair tiles: sums of n products of unit normal numbers, compensated FP32
+# (1e-6 of sum |x y|, the bound of the other Gram checks).
+@pytest.mark.parametrize("nx,ny", [(1, 1), (4, 4), (5, 8), (8, 8), (9, 12), (12, 12)])
+@pytest.mark.parametrize("n", [128, 128 * 1023])
+def test_gram_split_tiles(nx, ny, n):
+    g = torch.Generator("cuda").manual_seed(nx * ny)
+    x = torch.randn((nx, n), dtype=torch.float32, device="cuda", generator=g)
+    y = torch.randn((ny, n), dtype=torch.float32, device="cuda", generator=g)
+    xy = torch.cat([x, y])
+    got = ed.ed_gram_f32(xy.data_ptr(), nx, xy[nx:].data_ptr(), ny, n, n, 0)
+    ref = (x.double() @ y.double().T).cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-6 * float((x.abs().double() @ y.abs().double().T).max())
