@@ -38,6 +38,7 @@
 #include <numeric>
 #include <vector>
 
+#include "cf.cuh"
 #include "ed_common.cuh"
 
 namespace ed {
@@ -528,22 +529,184 @@ __global__ void __launch_bounds__(128) k_sym_apply_c(const SymDev* __restrict__ 
 
 // out[iz] += coef * b0sq / (z - s (a_0 - E0) - b_1^2 / (z - s (a_1 - E0) - ...)), n levels, s = +1
 // for the electron part and -1 for the hole part (Eq. jacobi with the E0 shift); z = zr + i zi.
-__global__ void k_sym_cf_eval(const double* __restrict__ alpha, const double* __restrict__ beta, int n, double E0,
-                              double b0sq, double s, const double* __restrict__ zr, const double* __restrict__ zi,
-                              int nz, double coef, double2* __restrict__ out) {
-  for (int iz = blockIdx.x * blockDim.x + threadIdx.x; iz < nz; iz += gridDim.x * blockDim.x) {
-    double gr = 0.0, gi = 0.0;  // the tail 1 / (z - ...) built from the last level up
-    for (int j = n - 1; j >= 0; --j) {
-      const double b2 = j + 1 < n ? beta[j + 1] * beta[j + 1] : 0.0;
-      const double dr = zr[iz] - s * (alpha[j] - E0) - b2 * gr;
-      const double di = zi[iz] - b2 * gi;
-      const double den = dr * dr + di * di;
-      gr = dr / den;
-      gi = -di / den;
-    }
-    out[iz].x += coef * b0sq * gr;
-    out[iz].y += coef * b0sq * gi;
+constexpr int kSymEvalThreads = 64;
+__global__ void __launch_bounds__(kSymEvalThreads) k_sym_cf_eval(const double* __restrict__ alpha, const double* __restrict__ beta,
+                                                                 int n, double E0, double b0sq, double s,
+                                                                 const double* __restrict__ zr, const double* __restrict__ zi,
+                                                                 int nz, double coef, double2* __restrict__ out) {
+  __shared__ double2 sm[kCfChunk];
+  const int iz = blockIdx.x * kSymEvalThreads + threadIdx.x, i = min(iz, nz - 1);
+  const double2 g = cf_eval_block(alpha, beta, n, b0sq, make_double2(zr[i], zi[i]), E0, -s, sm, iz < nz);
+  if (iz < nz) {
+    out[iz].x += coef * g.x;
+    out[iz].y += coef * g.y;
   }
+}
+
+// ---- several continued fractions of one real irrep sector together -------------------------
+// The runs' vectors are interleaved, x[i R + r], and R lanes share a row, each with its own run: an
+// entry of the matrix (12 bytes) is read once for all runs, the R operands of an entry are one
+// contiguous gather, and no sum crosses lanes.  Vectors are kept unnormalized with their norms
+// (u_n = b_n v_n), so a level is two launches:
+//   y = (1 / b_n) H u_n - (b_n / b_{n-1}) u_{n-1},  a_n = <u_n, y> / b_n         (k_sym_multi_spmv)
+//   u_{n+1} = y - (a_n / b_n) u_n,                  b_{n+1} = |u_{n+1}|          (k_sym_multi_axpy)
+// FP64-bound: one multiply-add per entry and run.  6 runs of 183,000 states (3x4 cluster, C2v): 80 us
+// per level, against 6 x 45 us one run at a time with eight lanes per row and three launches.
+constexpr int kSymMaxRuns = 8;
+
+struct SymMultiCoef {  // [runs][stride] each
+  double* alpha;  // a_n
+  double* norm;   // b_n (b_0 = |phi|)
+  double* inv;    // 1 / b_n, 0 when b_n = 0
+  int stride;
+};
+
+// Sums v per run over the block (thread t: run t % R) into partial[blockIdx.x R + r]; the last
+// block adds the partials in order and thread r of its first R threads returns true with the sum.
+__device__ __forceinline__ bool sym_multi_sum(double& v, int R, double* __restrict__ partial, unsigned* ticket) {
+  __shared__ double sm[32 * kSymMaxRuns];
+  __shared__ bool s_last;
+  const int t = threadIdx.x, row = t / R;
+  auto tree = [&]() {
+    sm[t] = v;
+    __syncthreads();
+    for (int w = 16; w > 0; w >>= 1) {
+      if (row < w) sm[t] += sm[t + w * R];
+      __syncthreads();
+    }
+    v = sm[t];
+  };
+  tree();
+  if (t < R) {
+    partial[blockIdx.x * R + t] = v;
+    __threadfence();
+  }
+  __syncthreads();
+  if (t == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  double s0 = 0.0, s1 = 0.0;
+  int b = row;
+  for (; b + 32 < (int)gridDim.x; b += 64) {
+    s0 += __ldcg(partial + b * R + t % R);
+    s1 += __ldcg(partial + (b + 32) * R + t % R);
+  }
+  if (b < (int)gridDim.x) s0 += __ldcg(partial + b * R + t % R);
+  v = s0 + s1;
+  __syncthreads();
+  tree();
+  if (t == 0) *ticket = 0u;
+  return t < R;
+}
+
+__global__ void k_sym_multi_spmv(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                 const double* __restrict__ val, int64_t dim, int R, const double* __restrict__ U,
+                                 double* __restrict__ Y, int n, SymMultiCoef c, double* __restrict__ partial, unsigned* ticket) {
+  const int r = threadIdx.x % R;
+  const double* inv = c.inv + (int64_t)r * c.stride;
+  const double f = inv[n], g = n > 0 ? c.norm[(int64_t)r * c.stride + n] * inv[n - 1] : 0.0;
+  double dot = 0.0;
+  for (int64_t i = blockIdx.x * 32 + threadIdx.x / R; i < dim; i += gridDim.x * 32) {
+    const int64_t k1 = rowptr[i + 1];
+    double acc = 0.0;
+    for (int64_t k = rowptr[i]; k < k1; k += 4) {
+      double v[4], x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const bool in = k + q < k1;
+        v[q] = in ? __ldg(val + k + q) : 0.0;
+        x[q] = __ldg(U + (int64_t)__ldg(col + (in ? k + q : k)) * R + r);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (k + q < k1) acc = fma(v[q], x[q], acc);
+    }
+    const int64_t o = i * R + r;
+    const double y = n > 0 ? fma(f, acc, -g * Y[o]) : f * acc;
+    Y[o] = y;
+    dot = fma(U[o], y, dot);
+  }
+  if (sym_multi_sum(dot, R, partial, ticket)) c.alpha[(int64_t)r * c.stride + n] = dot * f;
+}
+
+__global__ void k_sym_multi_axpy(int64_t dim, int R, const double* __restrict__ U, double* __restrict__ Y, int n,
+                                 SymMultiCoef c, double* __restrict__ partial, unsigned* ticket) {
+  const int r = threadIdx.x % R;
+  const int64_t o0 = (int64_t)r * c.stride;
+  const double h = c.alpha[o0 + n] * c.inv[o0 + n];
+  double s = 0.0;
+  for (int64_t i = blockIdx.x * 32 + threadIdx.x / R; i < dim; i += gridDim.x * 32) {
+    const int64_t o = i * R + r;
+    const double v = fma(-h, U[o], Y[o]);
+    Y[o] = v;
+    s = fma(v, v, s);
+  }
+  if (sym_multi_sum(s, R, partial, ticket)) {
+    const double b = sqrt(fmax(s, 0.0));
+    c.norm[o0 + n + 1] = b;
+    c.inv[o0 + n + 1] = b > 0.0 ? 1.0 / b : 0.0;
+  }
+}
+
+// U[i R + r] = a_r[i] (+ b_r[i]); the norms b_0.
+struct SymMultiStart {
+  const double* a[kSymMaxRuns];
+  const double* b[kSymMaxRuns];
+};
+__global__ void k_sym_multi_start(int64_t dim, int R, SymMultiStart st, double* __restrict__ U, SymMultiCoef c,
+                                  double* __restrict__ partial, unsigned* ticket) {
+  const int r = threadIdx.x % R;
+  const double* a = st.a[r];
+  const double* b = st.b[r];
+  double s = 0.0;
+  for (int64_t i = blockIdx.x * 32 + threadIdx.x / R; i < dim; i += gridDim.x * 32) {
+    const double v = b ? a[i] + b[i] : a[i];
+    U[i * R + r] = v;
+    s = fma(v, v, s);
+  }
+  if (sym_multi_sum(s, R, partial, ticket)) {
+    const double nb = sqrt(fmax(s, 0.0));
+    c.norm[(int64_t)r * c.stride] = nb;
+    c.inv[(int64_t)r * c.stride] = nb > 0.0 ? 1.0 / nb : 0.0;
+  }
+}
+
+// Convergence check after n levels (forward form of cf.cuh): the largest change on the grid since
+// the last check (n0 levels) into maxd[r]; the first level in (n0, n] whose b vanishes into brk[r].
+__global__ void __launch_bounds__(kSymEvalThreads) k_sym_multi_check(SymMultiCoef c, int n0, int n, double E0, double s,
+                                                                     const double* __restrict__ zr, const double* __restrict__ zi,
+                                                                     int nz, double2* __restrict__ state,
+                                                                     double2* __restrict__ prev, double bmin,
+                                                                     unsigned long long* __restrict__ maxd, int* __restrict__ brk) {
+  __shared__ double2 sm[kCfChunk];
+  const int r = blockIdx.y, iz = blockIdx.x * kSymEvalThreads + threadIdx.x, i = min(iz, nz - 1);
+  const bool use = iz < nz;
+  const double* norm = c.norm + (int64_t)r * c.stride;
+  if (blockIdx.x == 0)
+    for (int j = n0 + 1 + threadIdx.x; j <= n; j += kSymEvalThreads)
+      if (!(norm[j] > bmin)) atomicMin(brk + r, j);
+  const int64_t o = (int64_t)r * nz + i, m = (int64_t)gridDim.y * nz;
+  CfForward st;
+  if (use && n0 > 0) {
+    st.a1 = state[o];
+    st.a0 = state[m + o];
+    st.b1 = state[2 * m + o];
+    st.b0 = state[3 * m + o];
+  }
+  cf_advance_block(st, c.alpha + (int64_t)r * c.stride, norm, n0, n, make_double2(zr[i], zi[i]), E0, -s, sm, use);
+  double mx = 0.0;
+  if (use) {
+    state[o] = st.a1;
+    state[m + o] = st.a0;
+    state[2 * m + o] = st.b1;
+    state[3 * m + o] = st.b0;
+    const double2 g = st.value(norm[0] * norm[0]), p = prev[o];
+    mx = hypot(g.x - p.x, g.y - p.y);
+    prev[o] = g;
+  }
+  for (int w = 16; w > 0; w >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, w));
+  if ((threadIdx.x & 31) == 0) atomicMax(maxd + r, (unsigned long long)__double_as_longlong(mx));
 }
 
 }  // namespace ed
@@ -851,7 +1014,7 @@ static int sym_cf(ed_sym& T, const double* phi, double E0, double s_eh, const De
     levels = n + 1;
     if ((n + 1) % kSymCfCheck == 0 || n + 1 == maxn) {
       ED_CUDA(cudaMemsetAsync(g1.p, 0, nz * sizeof(double2), s));
-      k_sym_cf_eval<<<(nz + 127) / 128, 128, 0, s>>>(alpha.p, beta.p, levels, E0, b0sq, s_eh, zr.p, zi.p, nz, 1.0, g1.p);
+      k_sym_cf_eval<<<(nz + kSymEvalThreads - 1) / kSymEvalThreads, kSymEvalThreads, 0, s>>>(alpha.p, beta.p, levels, E0, b0sq, s_eh, zr.p, zi.p, nz, 1.0, g1.p);
       ED_CHECK_LAUNCH();
       ED_CUDA(cudaMemcpyAsync(h1.data(), g1.p, nz * sizeof(double2), cudaMemcpyDeviceToHost, s));
       ED_CUDA(cudaMemcpyAsync(hb.data(), beta.p, (n + 2) * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -876,15 +1039,90 @@ static int sym_cf(ed_sym& T, const double* phi, double E0, double s_eh, const De
       have_prev = true;
     }
   }
-  k_sym_cf_eval<<<(nz + 127) / 128, 128, 0, s>>>(alpha.p, beta.p, levels, E0, b0sq, s_eh, zr.p, zi.p, nz, coef, out);
+  k_sym_cf_eval<<<(nz + kSymEvalThreads - 1) / kSymEvalThreads, kSymEvalThreads, 0, s>>>(alpha.p, beta.p, levels, E0, b0sq, s_eh, zr.p, zi.p, nz, coef, out);
   ED_CHECK_LAUNCH();
   ED_CUDA(cudaStreamSynchronize(s));
   return levels;
 }
 
-__global__ void k_sym_add(const double* __restrict__ x, const double* __restrict__ y, int64_t n, double* __restrict__ z) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    z[i] = x[i] + y[i];
+// The fractions of R (at most kSymMaxRuns) runs of one real sector, as sym_cf for each: run r starts
+// from st.a[r] (+ st.b[r]) and its fraction is added to out[r].  All runs advance until the last has
+// stopped; each fraction uses the levels at which its own run stopped.
+static void sym_cf_multi(ed_sym& T, int R, const SymMultiStart& st, double E0, double s_eh, const DevBuf<double>& zr,
+                         const DevBuf<double>& zi, int nz, double tol, double2* const* out, cudaStream_t s) {
+  const int64_t dim = T.dim;
+  const int maxn = (int)std::min<int64_t>(kSymCfMax, 2 * dim + 16);
+  const int threads = 32 * R, grid = (int)std::max<int64_t>(1, std::min<int64_t>((dim + 31) / 32, 152 * 4));
+  DevBuf<double> U0(dim * R), U1(dim * R), coef((size_t)3 * R * (maxn + 2)), part((size_t)grid * R);
+  DevBuf<unsigned> tk(1);
+  DevBuf<double2> state((size_t)4 * R * nz), prev((size_t)R * nz);
+  DevBuf<unsigned long long> res(2 * kSymMaxRuns);  // maxd, then brk (ints)
+  const int stride = maxn + 2;
+  SymMultiCoef c{coef.p, coef.p + (size_t)R * stride, coef.p + (size_t)2 * R * stride, stride};
+  unsigned long long* maxd = res.p;
+  int* brk = reinterpret_cast<int*>(res.p + kSymMaxRuns);
+  ED_CUDA(cudaMemsetAsync(tk.p, 0, sizeof(unsigned), s));
+  ED_CUDA(cudaMemsetAsync(prev.p, 0, prev.n * sizeof(double2), s));
+  k_sym_multi_start<<<grid, threads, 0, s>>>(dim, R, st, U0.p, c, part.p, tk.p);
+  ED_CHECK_LAUNCH();
+  double* u = U0.p;
+  double* y = U1.p;
+  int levels[kSymMaxRuns], quiet[kSymMaxRuns] = {};
+  bool active[kSymMaxRuns];
+  double b0[kSymMaxRuns];
+  ED_CUDA(cudaMemcpy2DAsync(b0, sizeof(double), c.norm, stride * sizeof(double), sizeof(double), R, cudaMemcpyDeviceToHost, s));
+  ED_CUDA(cudaStreamSynchronize(s));
+  int left = 0;
+  for (int r = 0; r < R; ++r) {
+    levels[r] = 0;
+    active[r] = b0[r] > 0.0;
+    left += active[r];
+  }
+  const double bmin = 1e-10 * std::max(1.0, std::fabs(E0));
+  int checked = 0;
+  for (int n = 0; n < maxn && left > 0; ++n) {
+    {
+      ProfScope ps_(K_HPSI, s, (double)T.nnz * 12.0 + (double)dim * 16.0 * R);
+      k_sym_multi_spmv<<<grid, threads, 0, s>>>(T.rowptr.p, T.col.p, T.val.p, dim, R, u, y, n, c, part.p, tk.p);
+      ED_CHECK_LAUNCH();
+    }
+    k_sym_multi_axpy<<<grid, threads, 0, s>>>(dim, R, u, y, n, c, part.p, tk.p);
+    ED_CHECK_LAUNCH();
+    std::swap(u, y);
+    if ((n + 1) % kSymCfCheck == 0 || n + 1 == maxn) {
+      unsigned long long h[2 * kSymMaxRuns];
+      int* hbrk = reinterpret_cast<int*>(h + kSymMaxRuns);
+      ED_CUDA(cudaMemsetAsync(maxd, 0, kSymMaxRuns * sizeof(unsigned long long), s));
+      ED_CUDA(cudaMemsetAsync(brk, 0x7f, kSymMaxRuns * sizeof(int), s));
+      k_sym_multi_check<<<dim3((nz + kSymEvalThreads - 1) / kSymEvalThreads, R), kSymEvalThreads, 0, s>>>(
+          c, checked, n + 1, E0, s_eh, zr.p, zi.p, nz, state.p, prev.p, bmin, maxd, brk);
+      ED_CHECK_LAUNCH();
+      ED_CUDA(cudaMemcpyAsync(h, res.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+      ED_CUDA(cudaStreamSynchronize(s));
+      for (int r = 0; r < R; ++r) {
+        if (!active[r]) continue;
+        levels[r] = n + 1;
+        double d;
+        std::memcpy(&d, h + r, sizeof(d));
+        if (hbrk[r] <= n + 1) {  // an invariant subspace: stop at the first vanishing b_j
+          levels[r] = hbrk[r];
+          active[r] = false;
+        } else {
+          quiet[r] = checked > 0 && d < tol ? quiet[r] + 1 : 0;
+          if (quiet[r] >= 2) active[r] = false;  // two successive checks below the tolerance
+        }
+        left -= !active[r];
+      }
+      checked = n + 1;
+    }
+  }
+  for (int r = 0; r < R; ++r) {
+    if (levels[r] == 0) continue;
+    k_sym_cf_eval<<<(nz + kSymEvalThreads - 1) / kSymEvalThreads, kSymEvalThreads, 0, s>>>(
+        c.alpha + (size_t)r * stride, c.norm + (size_t)r * stride, levels[r], E0, b0[r] * b0[r], s_eh, zr.p, zi.p, nz, 1.0, out[r]);
+    ED_CHECK_LAUNCH();
+  }
+  ED_CUDA(cudaStreamSynchronize(s));
 }
 
 // z = x + y (mode 0) or x + i y (mode 1) on n interleaved complex values
@@ -1163,7 +1401,9 @@ static void sym_green(ed_sym& S, const double* omega, int nz, double eta, int ax
     zr_h[i] = axis == ED_AXIS_MATSUBARA ? 0.0 : omega[i];
     zi_h[i] = axis == ED_AXIS_MATSUBARA ? omega[i] : eta;
   }
-  DevBuf<double> zr(nz), zi(nz), Md(L);
+  DevBuf<double> zr(nz), zi(nz), Md((size_t)nrow * L);
+  for (int r = 0; r < nrow; ++r)
+    ED_CUDA(cudaMemcpyAsync(Md.p + (size_t)r * L, row_m[r].data(), L * sizeof(double), cudaMemcpyHostToDevice, s));
   ED_CUDA(cudaMemcpyAsync(zr.p, zr_h.data(), nz * sizeof(double), cudaMemcpyHostToDevice, s));
   ED_CUDA(cudaMemcpyAsync(zi.p, zi_h.data(), nz * sizeof(double), cudaMemcpyHostToDevice, s));
   std::vector<int> pidx(nrow * nrow, -1);
@@ -1192,22 +1432,35 @@ static void sym_green(ed_sym& S, const double* omega, int nz, double eta, int ax
       tgt[r] = T.get();
       if (T->dim == 0) continue;
       phi[r].alloc(T->dim);
-      ED_CUDA(cudaMemcpyAsync(Md.p, row_m[r].data(), L * sizeof(double), cudaMemcpyHostToDevice, s));
       k_sym_apply<<<sym_grid(T->dim, 128), 128, 0, s>>>(S.G.p, S.keys.p, S.stab.p, S.dim, S.omega.p, T->keys.p,
-                                                        T->stab.p, T->dim, Md.p, part == 0 ? 1 : 0, spin, phi[r].p);
+                                                        T->stab.p, T->dim, Md.p + (size_t)r * L, part == 0 ? 1 : 0, spin,
+                                                        phi[r].p);
       ED_CHECK_LAUNCH();
-      ED_CUDA(cudaStreamSynchronize(s));  // Md is rewritten for the next row
-      sym_cf(*T, phi[r].p, E0, s_eh, zr, zi, nz, tol, 1.0, D.p + (size_t)r * nz, s);
     }
-    for (int r = 0; r < nrow; ++r)
-      for (int q = r + 1; q < nrow; ++q) {
-        const int k = pidx[r * nrow + q];
-        if (k < 0 || tgt[r]->dim == 0) continue;
-        DevBuf<double> sum(tgt[r]->dim);
-        k_sym_add<<<sym_grid(tgt[r]->dim, kSymThreads * 4), kSymThreads, 0, s>>>(phi[r].p, phi[q].p, tgt[r]->dim, sum.p);
-        ED_CHECK_LAUNCH();
-        sym_cf(*tgt[r], sum.p, E0, s_eh, zr, zi, nz, tol, 1.0, P.p + (size_t)k * nz, s);
-      }
+    // the runs of every sector, at most kSymMaxRuns together: the rows' own, then the pairs'
+    for (auto& sec : sectors) {
+      ed_sym* T = sec.second.get();
+      if (T->dim == 0) continue;
+      SymMultiStart st = {};
+      double2* out[kSymMaxRuns];
+      int R = 0;
+      auto flush = [&]() {
+        if (R) sym_cf_multi(*T, R, st, E0, s_eh, zr, zi, nz, tol, out, s);
+        R = 0;
+      };
+      auto add = [&](const double* x, const double* y, double2* o) {
+        st.a[R] = x;
+        st.b[R] = y;
+        out[R] = o;
+        if (++R == kSymMaxRuns) flush();
+      };
+      for (int r = 0; r < nrow; ++r)
+        if (tgt[r] == T) add(phi[r].p, nullptr, D.p + (size_t)r * nz);
+      for (int r = 0; r < nrow; ++r)
+        for (int q = r + 1; q < nrow; ++q)
+          if (tgt[r] == T && pidx[r * nrow + q] >= 0) add(phi[r].p, phi[q].p, P.p + (size_t)pidx[r * nrow + q] * nz);
+      flush();
+    }
   }
   std::vector<double> Mh((size_t)nrow * ns);
   for (int r = 0; r < nrow; ++r)
