@@ -96,8 +96,12 @@ double* pinned_scratch();
 // the kernel's static shared memory).  Every caller sets the same value, so threads that launch
 // the kernel with different sizes at the same time (the server's lanes) cannot undo each other's
 // setting between setting it and launching.
+// Launches that fit the default limit (48 KB with a few KB of static shared memory) need no such call:
+// bytes = the launch's dynamic shared memory.  The attribute calls take about 3 us of host time, a fifth
+// of a small product.
 template <typename K>
-inline void allow_max_dynamic_smem(K* fn) {
+inline void allow_max_dynamic_smem(K* fn, size_t bytes = SIZE_MAX) {
+  if (bytes <= 40 * 1024) return;
   int dev = 0, optin = 0;
   ED_CUDA(cudaGetDevice(&dev));
   ED_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -172,6 +176,8 @@ struct HopParams {
   float u0f;
 };
 
+struct LineTables;  // lines64.cu
+
 // One spin's sector with N particles: basis, two-level rank tables, hopping table, diagonal.
 struct SpinTables {
   int L = 0, N = 0, split = 0;
@@ -185,6 +191,7 @@ struct SpinTables {
   DevBuf<uint32_t> ell;        // [zmax][dim] slot-major copy: ell[k * dim + r] = k-th entry of row r
   DevBuf<double> ediag;        // [dim] sum_a h_aa n_a
   DevBuf<float> ediag32;       // [dim]
+  std::shared_ptr<LineTables> lines;  // hops by magnitude (lines64.cu), built on first use
 };
 
 // Read-only device view of a two-spin sector for the H.psi kernels.
@@ -202,6 +209,10 @@ struct SectorView {
   const float* e_up32;
   const float* e_dn32;
   int zmax_up;              // most hops of an up-spin state
+  SpinTables* tab_up;       // the tables themselves, their model and the stream they are built on
+  SpinTables* tab_dn;
+  const ModelHost* model;
+  cudaStream_t tab_stream;
   int64_t two_pass_min_bytes;  // vectors of at least this many bytes take the two-pass H.psi
 };
 
@@ -273,6 +284,12 @@ void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, c
                          int nblk_cap, cudaStream_t s);
 int lanczos_blocks(const SectorView& sv);   // partial-sum slots per run of the fused step
 int two_pass_blocks(const SectorView& sv, int dtype);
+
+// lines64.cu: FP64 products with integer hop sums.
+bool lines64_usable(const SectorView& sv, cudaStream_t s);
+int lines64_blocks(const SectorView& sv);
+void launch_lines64(const SectorView& sv, const HopParams& hp, const double* X, double* O, int64_t vstride, int runs,
+                    const double* beta, int beta_stride, int n, const LanczosScalars* ls, cudaStream_t s);
 
 // small.cu: many Lanczos levels of small sectors in one launch, a thread-block cluster per run.
 struct SmallStore {  // where the vectors v_{n0 + 1}, v_{n0 + 2}, ... are kept too

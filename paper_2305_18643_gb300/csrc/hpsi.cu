@@ -684,6 +684,8 @@ static TilePlan tile_plan(const SectorView& sv, int dtype) {
   for (int tu : {4, 2, 1}) {
     const size_t smem = ((size_t)sv.d_dn * tu * es + 15) / 16 * 16 + (size_t)tu * p.zup * 16;
     if (smem > limit) continue;
+    // small sectors: fewer rows per tile rather than idle SMs
+    if (tu > 1 && (sv.d_up + tu - 1) / tu * ((sv.d_dn + 255) / 256) < 2 * 152) continue;
     p.tu = tu;
     p.smem = smem;
     break;
@@ -711,10 +713,10 @@ static void launch_tile(const TilePlan& p, const SectorView& sv, const HopParams
                         int runs, int n, const LanczosScalars* ls, cudaStream_t s) {
   const dim3 g((unsigned)std::min<int64_t>(p.units, kOnePassBlocks), runs);
   if (ls) {
-    allow_max_dynamic_smem(k_hpsi_tile<T, TU, true>);
+    allow_max_dynamic_smem(k_hpsi_tile<T, TU, true>, p.smem);
     k_hpsi_tile<T, TU, true><<<g, p.threads, p.smem, s>>>(sv, hp, X, O, vstride, p.nchunk, p.chunk, p.zup, n, *ls);
   } else {
-    allow_max_dynamic_smem(k_hpsi_tile<T, TU, false>);
+    allow_max_dynamic_smem(k_hpsi_tile<T, TU, false>, p.smem);
     k_hpsi_tile<T, TU, false><<<g, p.threads, p.smem, s>>>(sv, hp, X, O, vstride, p.nchunk, p.chunk, p.zup, n,
                                                           LanczosScalars{});
   }
@@ -754,7 +756,7 @@ static int one_pass_blocks(const SectorView& sv, int dtype) {
 
 int lanczos_blocks(const SectorView& sv) {
   // capacity for every form (the two-pass column kernel has the most blocks on large sectors)
-  return std::max({one_pass_blocks(sv, ED_FP64), one_pass_blocks(sv, ED_FP32), two_pass_blocks(sv, ED_FP64)});
+  return std::max({one_pass_blocks(sv, ED_FP64), one_pass_blocks(sv, ED_FP32), two_pass_blocks(sv, ED_FP64), lines64_blocks(sv)});
 }
 
 void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const void* x, void* y, cudaStream_t s) {
@@ -763,6 +765,10 @@ void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const voi
 
 void launch_hpsi_block(const SectorView& sv, const HopParams& hp, int dtype, const void* X, void* Y, int64_t vstride,
                        int runs, cudaStream_t s) {
+  if (dtype == ED_FP64 && lines64_usable(sv, s)) {
+    launch_lines64(sv, hp, (const double*)X, (double*)Y, vstride, runs, nullptr, 0, 0, nullptr, s);
+    return;
+  }
   const bool two = use_two_pass(sv, dtype, X, Y, vstride);
   if (dtype == ED_FP64) {
     if (two)
@@ -779,6 +785,11 @@ void launch_hpsi_block(const SectorView& sv, const HopParams& hp, int dtype, con
 
 void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, const void* X, void* XP,
                          int64_t vstride, int runs, int n, const LanczosScalars& ls, int nblk_cap, cudaStream_t s) {
+  if (dtype == ED_FP64 && lines64_usable(sv, s)) {
+    if (lines64_blocks(sv) > nblk_cap) throw Error(ED_ERR_INVALID, "partial buffer too small");
+    launch_lines64(sv, hp, (const double*)X, (double*)XP, vstride, runs, ls.beta, ls.mstride + 1, n, &ls, s);
+    return;
+  }
   const bool two = use_two_pass(sv, dtype, X, XP, vstride);
   if ((two ? two_pass_blocks(sv, dtype) : one_pass_blocks(sv, dtype)) > nblk_cap) throw Error(ED_ERR_INVALID, "partial buffer too small");
   if (dtype == ED_FP64) {

@@ -181,3 +181,45 @@ def test_gram_split_tiles(nx, ny, n):
     got = ed.ed_gram_f32(xy.data_ptr(), nx, xy[nx:].data_ptr(), ny, n, n, 0)
     ref = (x.double() @ y.double().T).cpu().numpy()
     assert np.abs(got - ref).max() <= 1e-6 * float((x.abs().double() @ y.abs().double().T).max())
+
+
+# FP64 products with integer hop sums (sectors of 2^19 states and more with few hop magnitudes): odd
+# dimensions and leading dimensions, and lines that leave the fixed point for the FP64 sums: one huge
+# element, zero and denormal rows, a row scaled to 1e-290.  Every row within 1e-12 of the largest |H| |x| that
+# feeds it, so small rows are held to their own scale.
+@pytest.mark.parametrize("W_,n_up,n_dn", [(7, 6, 7), (6, 6, 7), (7, 8, 5)])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_integer_hop_sums(W_, n_up, n_dn, pad):
+    rng = np.random.default_rng(W_ + n_up)
+    L = 2 * W_ + (1 if W_ == 6 else 0)
+    if W_ == 6:  # 13-site chain, one magnitude
+        c = W.random_cluster(rng, L, 0, n_up, n_dn, U=4.0)
+    else:
+        c = W.served_request(rng, sizes=(L,))
+        c = dict(c, n_up=n_up, n_dn=n_dn, U=c["U"] if pad else rng.uniform(1, 9, L))
+    op = O.sector_hamiltonian(_model(c), n_up, n_dn)
+    with ed.Cluster(c) as cl:
+        du, dd = ed.ed_sector_dims(cl.h, n_up, n_dn)
+        x = rng.standard_normal((du, dd))
+        x[3, 5] = 1e9
+        x[7] = 0.0
+        x[8] = 5e-310
+        x[9] *= 1e-290
+        xd = torch.zeros((du, dd + pad), dtype=torch.float64, device="cuda")
+        xd[:, :dd] = torch.tensor(x, device="cuda")
+        y = torch.full((du, dd + pad), 7.0, dtype=torch.float64, device="cuda")
+        args = (cl.h, n_up, n_dn, ed.ED_FP64, xd.data_ptr(), y.data_ptr(), dd + pad, torch.cuda.current_stream().cuda_stream)
+        ed.ed_hpsi(*args)
+        got = y.cpu().numpy()
+        xd[11, 2] = float("nan")
+        xd[13, 4] = float("inf")
+        ed.ed_hpsi(*args)
+        bad = ~np.isfinite(y[:, :dd].cpu().numpy())
+    ref = O.apply_h(op, x).reshape(du, dd)
+    fed = O.apply_h(op, (np.abs(x) > 1e5) * 1.0).reshape(du, dd) != 0.0  # rows and columns of the huge element
+    assert np.abs(got[:, :dd] - ref)[~fed].max() <= 1e-12 * np.abs(ref[~fed]).max()
+    assert np.abs(got[:, :dd] - ref)[fed].max() <= 1e-12 * np.abs(ref).max()
+    assert np.all(got[:, dd:] == 7.0)
+    z = np.zeros((du, dd))
+    z[11, 2] = z[13, 4] = 1.0
+    assert np.array_equal(bad, (O.apply_h(op, z).reshape(du, dd) != 0.0) | (z != 0.0))
