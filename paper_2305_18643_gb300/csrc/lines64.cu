@@ -24,6 +24,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "bank_order.cuh"
 #include "ed_common.cuh"
 #include "hpsi_element.cuh"
 
@@ -65,65 +66,14 @@ __global__ void k_line_fill(int64_t dim, const int32_t* __restrict__ ptr, const 
   const int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 8;
   if (r0 >= dim) return;
   const int nr = (int)(dim - r0 < 8 ? dim - r0 : 8);
-  unsigned long long left[8][4];  // entries of the row still to place (bit i: ptr + i), rows hold at most 256
-  unsigned long long res[8];      // number left per residue, a byte each
-  int nleft[8];
-  for (int i = 0; i < 8; ++i) {
-    for (int w = 0; w < 4; ++w) left[i][w] = 0ull;
-    res[i] = 0ull;
-    nleft[i] = 0;
-    if (i >= nr) continue;
-    const int32_t p0 = ptr[r0 + i], n = ptr[r0 + i + 1] - p0;
+  for (int i = 0; i < nr; ++i) {
+    const int n = ptr[r0 + i + 1] - ptr[r0 + i];
     cnt[r0 + i] = (uint8_t)n;
-    for (int k = 0; k < n; ++k) {
-      const uint32_t e = ent[p0 + k];
-      left[i][k >> 6] |= 1ull << (k & 63);
-      res[i] += 1ull << (8 * (ent_col(e) & 7u));
-      ++nleft[i];
-    }
     for (int k = n; k < slots; ++k) ell[(int64_t)k * dim + r0 + i] = (uint32_t)dim << 4;
   }
-  for (int slot = 0;; ++slot) {
-    unsigned freebank = 0xffu, todo = 0u;
-    for (int i = 0; i < nr; ++i)
-      if (nleft[i] > 0) todo |= 1u << i;
-    if (!todo) break;
-    while (todo) {
-      int i = -1;
-      for (int q = 0; q < nr; ++q)
-        if ((todo >> q & 1u) && (i < 0 || nleft[q] > nleft[i])) i = q;
-      todo &= ~(1u << i);
-      int bank = -1, best = 0, any = -1;
-      for (int b = 0; b < 8; ++b) {
-        const int c = (int)(res[i] >> (8 * b) & 0xffull);
-        if (c > 0 && any < 0) any = b;
-        if (c > best && (freebank >> b & 1u)) {
-          best = c;
-          bank = b;
-        }
-      }
-      if (bank < 0) bank = any;
-      freebank &= ~(1u << bank);
-      const int32_t p0 = ptr[r0 + i];
-      for (int w = 0; w < 4; ++w) {
-        unsigned long long m = left[i][w];
-        bool hit = false;
-        while (m) {
-          const int k = w * 64 + __ffsll((long long)m) - 1;
-          m &= m - 1ull;
-          const uint32_t e = ent[p0 + k];
-          if ((int)(ent_col(e) & 7u) != bank) continue;
-          left[i][w] &= ~(1ull << (k & 63));
-          ell[(int64_t)slot * dim + r0 + i] = (ent_col(e) << 4) | (cm.of[ent_vidx(e)] ^ ent_neg(e));
-          hit = true;
-          break;
-        }
-        if (hit) break;
-      }
-      res[i] -= 1ull << (8 * bank);
-      --nleft[i];
-    }
-  }
+  bank_order_group(ptr, ent, r0, nr, [&](int slot, int i, uint32_t e) {
+    ell[(int64_t)slot * dim + r0 + i] = (ent_col(e) << 4) | (cm.of[ent_vidx(e)] ^ ent_neg(e));
+  });
 }
 
 // Builds the table of one spin.

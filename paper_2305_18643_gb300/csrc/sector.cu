@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "bank_order.cuh"
 #include "ed_common.cuh"
 
 namespace ed {
@@ -176,86 +177,17 @@ __global__ void k_ediag(int64_t dim, int L, const uint32_t* __restrict__ basis, 
 
 static inline unsigned nblocks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// Slot-major copy of the CSR table (ell[k * dim + r] = an entry of row r, 0 past its end) whose
-// order within each row is chosen against shared-memory bank conflicts of the row kernel: there,
-// the threads of rows 8m .. 8m+7 gather 16-byte words sx[col] together at every slot, and a
-// 16-byte load of 8 threads takes one shared-memory wavefront when their col mod 8 differ.  Per
-// group of 8 rows and per slot, a maximum matching of the rows that still have entries to the
-// eight residues col mod 8 (augmenting paths; rows with more remaining entries first, each row
-// trying its most frequent residues first) picks one entry per matched row; unmatched rows take
-// their first remaining entry.  Every row keeps its entry set, so only the order of the
-// additions changes.
+// Slot-major copy of the CSR table whose order within each row is chosen against shared-memory bank
+// conflicts of the row kernel (bank_order.cuh), for sectors that can reach that kernel's sizes.
 constexpr int64_t kEllOrderMinDim = 2048;
+constexpr int kOrderThreads = 32;
 
-namespace {
-struct BankMatch {
-  std::vector<uint32_t>* rem;  // [8] remaining entries of each row
-  int owner[8];                // residue -> row (-1 free)
-  bool seen[8];
-  bool augment(int i) {
-    int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (uint32_t e : rem[i]) ++cnt[ent_col(e) & 7u];
-    for (int pass = 0; pass < 8; ++pass) {
-      int r = -1;
-      for (int k = 0; k < 8; ++k)
-        if (cnt[k] > 0 && !seen[k] && (r < 0 || cnt[k] > cnt[r])) r = k;
-      if (r < 0) return false;
-      seen[r] = true;
-      cnt[r] = 0;
-      if (owner[r] < 0 || augment(owner[r])) {
-        owner[r] = i;
-        return true;
-      }
-    }
-    return false;
-  }
-};
-}  // namespace
-
-static void ell_bank_order(const std::vector<int32_t>& ptr, const std::vector<uint32_t>& ent, int64_t dim, int zmax,
-                           std::vector<uint32_t>& ell) {
-  ell.assign((size_t)zmax * dim, 0u);
-  std::vector<uint32_t> rem[8];
-  BankMatch bm;
-  bm.rem = rem;
-  for (int64_t r0 = 0; r0 < dim; r0 += 8) {
-    const int nr = (int)std::min<int64_t>(8, dim - r0);
-    for (int i = 0; i < 8; ++i) {
-      if (i < nr)
-        rem[i].assign(ent.begin() + ptr[r0 + i], ent.begin() + ptr[r0 + i + 1]);
-      else
-        rem[i].clear();
-    }
-    for (int k = 0;; ++k) {
-      int order[8], na = 0;
-      for (int i = 0; i < nr; ++i)
-        if (!rem[i].empty()) order[na++] = i;
-      if (na == 0) break;
-      std::sort(order, order + na, [&](int a, int b) { return rem[a].size() > rem[b].size(); });
-      for (int r = 0; r < 8; ++r) bm.owner[r] = -1;
-      for (int oi = 0; oi < na; ++oi) {
-        for (int r = 0; r < 8; ++r) bm.seen[r] = false;
-        bm.augment(order[oi]);
-      }
-      int res_of[8];
-      for (int i = 0; i < 8; ++i) res_of[i] = -1;
-      for (int r = 0; r < 8; ++r)
-        if (bm.owner[r] >= 0) res_of[bm.owner[r]] = r;
-      for (int oi = 0; oi < na; ++oi) {
-        const int i = order[oi];
-        auto& v = rem[i];
-        size_t pick = 0;
-        if (res_of[i] >= 0)
-          for (size_t j = 0; j < v.size(); ++j)
-            if ((int)(ent_col(v[j]) & 7u) == res_of[i]) {
-              pick = j;
-              break;
-            }
-        ell[(size_t)k * dim + r0 + i] = row_ell_pack(v[pick]);
-        v.erase(v.begin() + (ptrdiff_t)pick);
-      }
-    }
-  }
+__global__ void __launch_bounds__(kOrderThreads) k_ell_order(int64_t dim, const int32_t* __restrict__ ptr,
+                                                             const uint32_t* __restrict__ ent, uint32_t* __restrict__ ell) {
+  const int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 8;
+  if (r0 >= dim) return;
+  bank_order_group(ptr, ent, r0, (int)(dim - r0 < 8 ? dim - r0 : 8),
+                   [&](int slot, int i, uint32_t e) { ell[(int64_t)slot * dim + r0 + i] = row_ell_pack(e); });
 }
 
 std::unique_ptr<SpinTables> build_spin_tables(const ModelHost& m, int N, cudaStream_t s) {
@@ -322,16 +254,9 @@ std::unique_ptr<SpinTables> build_spin_tables(const ModelHost& m, int N, cudaStr
     t->ell.alloc(std::max<int64_t>((int64_t)(t->zmax + kEllPad) * dim, 1));
     ED_CUDA(cudaMemsetAsync(t->ell.p, 0, (size_t)(t->zmax + kEllPad) * dim * sizeof(uint32_t), s));
     if (dim >= kEllOrderMinDim && t->zmax > 0) {
-      // large sectors: slot order chosen on the host against shared-memory bank conflicts
-      std::vector<int32_t> hptr(dim + 1);
-      std::vector<uint32_t> hent(std::max<int64_t>(nnz, 1));
-      ED_CUDA(cudaMemcpyAsync(hptr.data(), t->ptr.p, (dim + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-      ED_CUDA(cudaMemcpyAsync(hent.data(), t->ent.p, std::max<int64_t>(nnz, 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-      ED_CUDA(cudaStreamSynchronize(s));
-      std::vector<uint32_t> hell;
-      ell_bank_order(hptr, hent, dim, t->zmax, hell);
-      ED_CUDA(cudaMemcpyAsync(t->ell.p, hell.data(), hell.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
-      ED_CUDA(cudaStreamSynchronize(s));
+      ProfScope ps_(K_TABLES, s, 0.0);
+      k_ell_order<<<nblocks((dim + 7) / 8, kOrderThreads), kOrderThreads, 0, s>>>(dim, t->ptr.p, t->ent.p, t->ell.p);
+      ED_CHECK_LAUNCH();
     } else if (dim > 0 && t->zmax > 0) {
       { ProfScope ps_(K_TABLES, s, 0.0); k_ell_fill<<<nblocks(dim, bs), bs, 0, s>>>(dim, t->ptr.p, t->ent.p, t->zmax, t->ell.p); }
       ED_CHECK_LAUNCH();

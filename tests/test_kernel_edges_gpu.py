@@ -223,3 +223,27 @@ def test_integer_hop_sums(W_, n_up, n_dn, pad):
     z = np.zeros((du, dd))
     z[11, 2] = z[13, 4] = 1.0
     assert np.array_equal(bad, (O.apply_h(op, z).reshape(du, dd) != 0.0) | (z != 0.0))
+
+
+# The two-pass kernels on tables ordered on the device (from 2,048 states per spin), with few and with
+# many hop values (FP64: more than four magnitudes keep them off the integer sums).
+@pytest.mark.parametrize("dtype,many", [(torch.float32, False), (torch.float32, True), (torch.float64, True)])
+@pytest.mark.parametrize("n_up,n_dn", [(7, 7), (5, 8)])
+def test_two_pass_ordered_tables(dtype, many, n_up, n_dn):
+    rng = np.random.default_rng(n_up)
+    c = W.served_request(rng, sizes=(14,))
+    t = c["t"] * np.triu(rng.uniform(0.5, 1.5, c["t"].shape), 1) if many else np.triu(c["t"], 1)
+    c = dict(c, t=t + t.T, n_up=n_up, n_dn=n_dn)
+    op = O.sector_hamiltonian(_model(c), n_up, n_dn)
+    with ed.Cluster(c) as cl:
+        du, dd = ed.ed_sector_dims(cl.h, n_up, n_dn)
+        ld = (dd + 127) // 128 * 128
+        x = torch.zeros((du, ld), dtype=dtype, device="cuda")
+        x[:, :dd] = torch.tensor(rng.standard_normal((du, dd)), device="cuda")
+        y = torch.zeros_like(x)
+        ed.ed_hpsi(cl.h, n_up, n_dn, ed.ED_FP64 if dtype == torch.float64 else ed.ED_FP32, x.data_ptr(), y.data_ptr(), ld,
+                   torch.cuda.current_stream().cuda_stream)
+        got = y.cpu().double().numpy()
+    ref = O.apply_h(op, x[:, :dd].cpu().double().numpy()).reshape(du, dd)
+    assert np.abs(got[:, :dd] - ref).max() <= (1e-12 if dtype == torch.float64 else 2e-5) * np.abs(ref).max()
+    assert np.all(got[:, dd:] == 0.0)
