@@ -2,6 +2,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -11,6 +13,41 @@ namespace ed {
 
 static thread_local std::string g_last_error;
 thread_local cudaStream_t g_alloc_stream = nullptr;
+thread_local cudaMemPool_t g_alloc_pool = nullptr;
+
+namespace {
+std::mutex g_pools_mu;
+std::map<int, cudaMemPool_t> g_pools;
+}  // namespace
+
+cudaMemPool_t device_pool() {
+  int dev = 0;
+  ED_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(g_pools_mu);
+  auto it = g_pools.find(dev);
+  if (it != g_pools.end()) return it->second;
+  cudaMemPool_t pool = nullptr;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+    uint64_t keep = kPoolKeep;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  } else {
+    cudaGetLastError();
+    pool = nullptr;
+  }
+  return g_pools[dev] = pool;
+}
+
+void trim_device_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lk(g_pools_mu);
+  auto it = g_pools.find(dev);
+  if (it != g_pools.end() && it->second) cudaMemPoolTrimTo(it->second, 0);
+}
 
 namespace {
 struct PinnedScratch {
@@ -180,6 +217,7 @@ SpinTables& ed_cluster::tables(int N) {
   auto it = spins.find(N);
   if (it != spins.end()) return *it->second;
   if (N < 0 || N > model.L) throw Error(ED_ERR_INVALID, "particle number outside [0, L]");
+  PlainAllocScope plain;  // the tables are read on any stream
   auto t = build_spin_tables(model, N, stream);
   SpinTables& ref = *t;
   spins[N] = std::move(t);
@@ -241,6 +279,7 @@ ed_status ed_ground_state(ed_cluster* c, double* E0, double* residual, int* iter
   return guarded([&]() -> ed_status {
     require(c != nullptr, "cluster is NULL");
     require_cluster_device(c);
+    PoolScope pool(c->owns_stream ? c->stream : nullptr);
     GroundResult r;
     if (c->davidson_states > 1) {
       LowStatesResult d = run_davidson(*c, c->davidson_states, c->desc.tol, c->desc.max_iter, c->desc.seed);
@@ -288,6 +327,7 @@ ed_status ed_green(ed_cluster* c, const double* omega, int n_freq, double eta, i
     require(spin == 0 || spin == 1, "spin must be 0 or 1");
     require(is_finite(eta), "eta is not finite");
     require_cluster_device(c);
+    PoolScope pool(c->owns_stream ? c->stream : nullptr);
     ed_status st = ED_OK;
     if (!c->have_gs) {
       st = ed_ground_state(c, nullptr, nullptr, nullptr);

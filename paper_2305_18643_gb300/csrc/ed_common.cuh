@@ -86,6 +86,52 @@ struct AllocStreamScope {
   AllocStreamScope& operator=(const AllocStreamScope&) = delete;
 };
 
+// Memory of one solve (ground state, Green function) of a cluster with a stream of its own: DevBufs come
+// stream-ordered from a pool of the library, one per device, that keeps at most kPoolKeep bytes between
+// calls and returns the rest to the device when a stream is synchronized (and those too when an allocation
+// of the library finds no memory).  cudaMalloc and cudaFree (which
+// waits for the device) took 4 ms of a 55 ms solve and most of a small one.  Only buffers used on the
+// cluster's stream alone may come from it: the sector tables, which ed_hpsi reads on the caller's stream,
+// are allocated under PlainAllocScope.  Nested scopes (the server's lanes) keep the outer one.  Buffers
+// beyond kPoolMaxAlloc stay with cudaMalloc: the pool would hand them back at every synchronization.
+constexpr size_t kPoolMaxAlloc = size_t(256) << 20;
+constexpr size_t kPoolKeep = size_t(4) << 30;
+extern thread_local cudaMemPool_t g_alloc_pool;
+cudaMemPool_t device_pool();  // the current device's pool; nullptr when the device has none
+void trim_device_pool();      // returns what that pool holds unused to the device
+struct PoolScope {
+  cudaStream_t prev_s;
+  cudaMemPool_t prev_p;
+  explicit PoolScope(cudaStream_t s) : prev_s(g_alloc_stream), prev_p(g_alloc_pool) {
+    if (!g_alloc_stream && s) {
+      g_alloc_pool = device_pool();
+      if (g_alloc_pool) g_alloc_stream = s;
+    }
+  }
+  ~PoolScope() {
+    g_alloc_stream = prev_s;
+    g_alloc_pool = prev_p;
+  }
+  PoolScope(const PoolScope&) = delete;
+  PoolScope& operator=(const PoolScope&) = delete;
+};
+struct PlainAllocScope {  // plain cudaMalloc inside a PoolScope
+  cudaStream_t prev_s;
+  cudaMemPool_t prev_p;
+  PlainAllocScope() : prev_s(g_alloc_stream), prev_p(g_alloc_pool) {
+    if (g_alloc_pool) {
+      g_alloc_stream = nullptr;
+      g_alloc_pool = nullptr;
+    }
+  }
+  ~PlainAllocScope() {
+    g_alloc_stream = prev_s;
+    g_alloc_pool = prev_p;
+  }
+  PlainAllocScope(const PlainAllocScope&) = delete;
+  PlainAllocScope& operator=(const PlainAllocScope&) = delete;
+};
+
 // Page-locked host scratch of this thread (kPinnedSlots doubles, allocated on first use and kept
 // for the thread's life), the landing place of small device-to-host reads.  Slots: [0, 16) ground
 // state, 16 continued fractions, 17 band Lanczos.
@@ -132,7 +178,26 @@ struct DevBuf {
     release();
     if (count == 0) return;
     cudaStream_t as = g_alloc_stream;
-    cudaError_t e = as ? cudaMallocAsync((void**)&p, count * sizeof(T), as) : cudaMalloc(&p, count * sizeof(T));
+    cudaError_t e;
+    if (as && g_alloc_pool && count * sizeof(T) > kPoolMaxAlloc) as = nullptr;
+    if (as && g_alloc_pool) {
+      e = cudaMallocFromPoolAsync((void**)&p, count * sizeof(T), g_alloc_pool, as);
+      if (e == cudaErrorMemoryAllocation) {  // return what the pool holds unused, and try once more
+        cudaGetLastError();
+        cudaStreamSynchronize(as);
+        trim_device_pool();
+        e = cudaMallocFromPoolAsync((void**)&p, count * sizeof(T), g_alloc_pool, as);
+      }
+    } else if (as) {
+      e = cudaMallocAsync((void**)&p, count * sizeof(T), as);
+    } else {
+      e = cudaMalloc(&p, count * sizeof(T));
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        trim_device_pool();
+        e = cudaMalloc(&p, count * sizeof(T));
+      }
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
@@ -194,8 +259,10 @@ struct SpinTables {
   std::shared_ptr<LineTables> lines;  // hops by magnitude (lines64.cu), built on first use
 };
 
-// Read-only device view of a two-spin sector for the H.psi kernels.
-struct SectorView {
+// Read-only device view of a two-spin sector for the H.psi kernels.  The two-pass kernels take these fields
+// alone: with the host's fields below among their parameters they were 1.2 % slower (2x7, FP32: 132.0 us a
+// product against 130.3; 4x4: 2202 us against 2172).
+struct SectorArgs {
   int64_t d_up, d_dn, ld;
   const uint32_t* B_up;
   const uint32_t* B_dn;
@@ -208,12 +275,16 @@ struct SectorView {
   const double* e_dn;
   const float* e_up32;
   const float* e_dn32;
+  int64_t two_pass_min_bytes;  // vectors of at least this many bytes take the two-pass H.psi
+};
+
+// With what only the host's choices need.
+struct SectorView : SectorArgs {
   int zmax_up;              // most hops of an up-spin state
   SpinTables* tab_up;       // the tables themselves, their model and the stream they are built on
   SpinTables* tab_dn;
   const ModelHost* model;
   cudaStream_t tab_stream;
-  int64_t two_pass_min_bytes;  // vectors of at least this many bytes take the two-pass H.psi
 };
 
 // Preset maximum of a continued fraction of the batched and served forms when the caller gives
@@ -269,6 +340,7 @@ struct LanczosScalars {
   int mstride;
   double btol;        // run stops when b_{n+1} < btol * b_0
   int* nsteps;        // [runs] levels completed (alpha_0 .. alpha_{nsteps-1}); may be NULL
+  const void* prev = nullptr;  // v_{n-1} of the fused step where it is not in the output buffer (one run)
 };
 
 void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const void* x, void* y,
@@ -278,7 +350,8 @@ void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const voi
 void launch_hpsi_block(const SectorView& sv, const HopParams& hp, int dtype, const void* X, void* Y, int64_t vstride,
                        int runs, cudaStream_t s);
 // One fused Lanczos step for `runs` vectors stored at X + r * vstride (and XP likewise):
-// W = H X - b_n XP written over XP; per-run reductions finish alpha_n, b_{n+1}.
+// W = H X - b_n XP written over XP (or, with ls.prev, W = H X - b_n prev written to XP); per-run reductions finish
+// alpha_n, b_{n+1}.
 void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, const void* X,
                          void* XP, int64_t vstride, int runs, int n, const LanczosScalars& ls,
                          int nblk_cap, cudaStream_t s);
@@ -301,10 +374,10 @@ void launch_small_levels(const SectorView& sv, const HopParams& hp, int dtype, v
                          int n0, int n1, const LanczosScalars& ls, int nb, const SmallStore& store, cudaStream_t s);
 
 // lanczos.cu
-// omega (contiguous) += coef[n + 1] v_{n+1}; its type is omega_dtype (< 0: the vectors' dtype).
+// v_{n+1} = (W - a_n X) / b_{n+1} over W, or to dst; omega (contiguous) += coef[n + 1] v_{n+1}; its type is omega_dtype (< 0: the vectors' dtype).
 void launch_lanczos_next(int dtype, void* W, const void* X, int64_t d_up, int64_t d_dn, int64_t ld,
                          int64_t vstride, int runs, int n, const LanczosScalars& ls,
-                         void* omega, const double* coef, cudaStream_t s, int omega_dtype = -1);
+                         void* omega, const double* coef, cudaStream_t s, int omega_dtype = -1, void* dst = nullptr);
 void launch_start_vector(int dtype, void* v, int64_t d_up, int64_t d_dn, int64_t ld, uint64_t seed,
                          cudaStream_t s);
 // Reductions into a device double: out = <a, b> over d_up x d_dn (two-stage, fixed order).

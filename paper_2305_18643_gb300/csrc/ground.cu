@@ -100,7 +100,7 @@ struct VectorStore {
     vbytes = vb;
     count = 0;
     chunks.clear();
-    ok = g_alloc_stream == nullptr;
+    ok = g_alloc_stream == nullptr || g_alloc_pool != nullptr;
   }
   char* at(int n) { return chunks[n / kChunk].p + (size_t)(n % kChunk) * vbytes; }
   void drop() {
@@ -108,31 +108,28 @@ struct VectorStore {
     chunks.clear();  // cudaFree waits for the copies in flight
     count = 0;
   }
-  void push(const void* src, cudaStream_t s) {
-    if (!ok) return;
+  // The slot of the next vector (row padding zeroed), or nullptr when it does not fit.
+  char* next(int64_t du, size_t row_bytes, size_t pad_bytes, cudaStream_t s) {
+    if (!ok) return nullptr;
     if (count == (int)chunks.size() * kChunk) {
       size_t fr = 0, tot = 0;
       if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
         cudaGetLastError();
-        drop();
-        return;
+        return nullptr;
       }
       const size_t need = (size_t)kChunk * vbytes;
-      if (fr < need + std::max<size_t>(tot / 4, size_t(8) << 30)) {
-        drop();
-        return;
-      }
+      if (fr < need + std::max<size_t>(tot / 4, size_t(8) << 30)) return nullptr;
       DevBuf<char> b;
       try {
         b.alloc(need);
       } catch (const Error&) {
-        drop();
-        return;
+        return nullptr;
       }
+      if (pad_bytes)
+        ED_CUDA(cudaMemset2DAsync(b.p + row_bytes, row_bytes + pad_bytes, 0, pad_bytes, (size_t)du * kChunk, s));
       chunks.push_back(std::move(b));
     }
-    ED_CUDA(cudaMemcpyAsync(at(count), src, vbytes, cudaMemcpyDeviceToDevice, s));
-    ++count;
+    return at(count++);
   }
 };
 
@@ -254,18 +251,36 @@ static int lanczos_pass(ed_cluster& c, const SectorView& sv, int dtype, LanczosR
     L.reset(s);
     ED_CUDA(cudaMemcpyAsync(V[0], Vstart, bytes, cudaMemcpyDeviceToDevice, s));
     ED_CUDA(cudaMemsetAsync(V[1], 0, bytes, s));
+    const size_t es = esize(dtype), row = (size_t)dd * es, pad = (size_t)(ld - dd) * es;
     if (pass == 0) {
       store.start(bytes);
-      store.push(V[0], s);
+      if (char* v = store.next(du, row, pad, s))
+        ED_CUDA(cudaMemcpyAsync(v, V[0], bytes, cudaMemcpyDeviceToDevice, s));
+      else
+        store.drop();
     }
     if (pass == 1) launch_copy_ld(dtype, omega, dd, dtype, V[0], ld, L.svec.p, du, dd, s);
     int cur = 0;
     const int nmax = pass == 0 ? L.M : m - 1;
     for (int n = 0; n < nmax; ++n) {
-      launch_lanczos_step(sv, c.hp, dtype, V[cur], V[cur ^ 1], 0, 1, n, L.ls, L.nblk, s);
-      launch_lanczos_next(dtype, V[cur ^ 1], V[cur], du, dd, ld, 0, 1, n, L.ls, pass == 1 ? omega : nullptr, L.svec.p, s);
-      if (pass == 0) store.push(V[cur ^ 1], s);
-      cur ^= 1;
+      char* v = pass == 0 ? store.next(du, row, pad, s) : nullptr;
+      if (pass == 0 && store.ok && !v) {  // no more room: the last two vectors go on in V, the rest is retraced
+        ED_CUDA(cudaMemcpyAsync(V[0], store.at(n), bytes, cudaMemcpyDeviceToDevice, s));
+        if (n > 0) ED_CUDA(cudaMemcpyAsync(V[1], store.at(n - 1), bytes, cudaMemcpyDeviceToDevice, s));
+        ED_CUDA(cudaStreamSynchronize(s));
+        store.drop();
+        cur = 0;
+      }
+      if (v) {  // v_{n+1} straight into its slot, w in V[0], v_n and v_{n-1} from theirs
+        LanczosScalars ls = L.ls;
+        ls.prev = n > 0 ? (const void*)store.at(n - 1) : V[1];
+        launch_lanczos_step(sv, c.hp, dtype, store.at(n), V[0], 0, 1, n, ls, L.nblk, s);
+        launch_lanczos_next(dtype, V[0], store.at(n), du, dd, ld, 0, 1, n, L.ls, nullptr, L.svec.p, s, -1, v);
+      } else {
+        launch_lanczos_step(sv, c.hp, dtype, V[cur], V[cur ^ 1], 0, 1, n, L.ls, L.nblk, s);
+        launch_lanczos_next(dtype, V[cur ^ 1], V[cur], du, dd, ld, 0, 1, n, L.ls, pass == 1 ? omega : nullptr, L.svec.p, s);
+        cur ^= 1;
+      }
       if (pass == 0 && ((n + 1) % kCheck == 0 || n + 1 == L.M)) {
         ED_CUDA(cudaMemcpyAsync(host + 8, L.active.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         ED_CUDA(cudaStreamSynchronize(s));
@@ -321,9 +336,13 @@ static int refine_round(ed_cluster& c, const SectorView& sv, LanczosRun& L, floa
     ED_CUDA(cudaMemcpyAsync(scal.p + 5, &inv, sizeof(double), cudaMemcpyHostToDevice, s));
     launch_copy_ld(ED_FP32, V[0], ld, ED_FP64, omega, dd, nullptr, du, dd, s);       // q_0
     launch_copy_ld(ED_FP32, V[1], ld, ED_FP64, r, dd, scal.p + 5, du, dd, s);        // q_1 = r / |r|
+    const size_t bytes = (size_t)du * ld * sizeof(float), row = (size_t)dd * sizeof(float), pad = (size_t)(ld - dd) * sizeof(float);
     if (pass == 0) {
-      store.start((size_t)du * ld * sizeof(float));
-      store.push(V[1], s);
+      store.start(bytes);
+      if (char* v = store.next(du, row, pad, s))
+        ED_CUDA(cudaMemcpyAsync(v, V[1], bytes, cudaMemcpyDeviceToDevice, s));
+      else
+        store.drop();
     }
     if (pass == 1) {
       // omega <- s_0 omega + (s_1 / |r|) r, in FP64; the loop adds s_n q_n for n >= 2
@@ -337,11 +356,26 @@ static int refine_round(ed_cluster& c, const SectorView& sv, LanczosRun& L, floa
     int cur = 1;
     const int nmax = pass == 0 ? L.M : m - 1;
     for (int n = 1; n < nmax; ++n) {
-      launch_lanczos_step(sv, c.hp, ED_FP32, V[cur], V[cur ^ 1], 0, 1, n, L.ls, L.nblk, s);
-      launch_lanczos_next(ED_FP32, V[cur ^ 1], V[cur], du, dd, ld, 0, 1, n, L.ls, pass == 1 ? omega : nullptr, L.svec.p,
-                          s, ED_FP64);
-      if (pass == 0) store.push(V[cur ^ 1], s);
-      cur ^= 1;
+      // slot k holds q_{k+1}
+      char* v = pass == 0 ? store.next(du, row, pad, s) : nullptr;
+      if (pass == 0 && store.ok && !v) {  // no more room, as in lanczos_pass
+        ED_CUDA(cudaMemcpyAsync(V[1], store.at(n - 1), bytes, cudaMemcpyDeviceToDevice, s));
+        if (n > 1) ED_CUDA(cudaMemcpyAsync(V[0], store.at(n - 2), bytes, cudaMemcpyDeviceToDevice, s));
+        ED_CUDA(cudaStreamSynchronize(s));
+        store.drop();
+        cur = 1;
+      }
+      if (v) {  // w in V[1], q_{n-1} from its slot (q_0 from V[0])
+        LanczosScalars ls = L.ls;
+        ls.prev = n > 1 ? (const void*)store.at(n - 2) : V[0];
+        launch_lanczos_step(sv, c.hp, ED_FP32, store.at(n - 1), V[1], 0, 1, n, ls, L.nblk, s);
+        launch_lanczos_next(ED_FP32, V[1], store.at(n - 1), du, dd, ld, 0, 1, n, L.ls, nullptr, L.svec.p, s, ED_FP64, v);
+      } else {
+        launch_lanczos_step(sv, c.hp, ED_FP32, V[cur], V[cur ^ 1], 0, 1, n, L.ls, L.nblk, s);
+        launch_lanczos_next(ED_FP32, V[cur ^ 1], V[cur], du, dd, ld, 0, 1, n, L.ls, pass == 1 ? omega : nullptr, L.svec.p, s,
+                            ED_FP64);
+        cur ^= 1;
+      }
       if (pass == 0 && ((n + 1) % kCheck == 0 || n + 1 == L.M)) {
         ED_CUDA(cudaMemcpyAsync(host + 8, L.active.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         ED_CUDA(cudaStreamSynchronize(s));

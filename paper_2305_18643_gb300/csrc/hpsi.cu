@@ -16,6 +16,7 @@
 // the device and repeated runs are bitwise identical.
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "ed_common.cuh"
 #include "hpsi_element.cuh"
@@ -85,13 +86,14 @@ __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams
   load_params<T>(hp, sval, sU);
   const T* X = X0 + run * vstride;
   T* O = O0 + run * vstride;
+  const T* P = FUSED && ls.prev ? (const T*)ls.prev : O;
   const T bn = FUSED ? (T)ls.beta[(int64_t)run * (ls.mstride + 1) + n] : T(0);
   double sxw = 0.0, sww = 0.0, sxx = 0.0;
   auto element = [&](int64_t u, int64_t d) {
     const int64_t o = u * sv.ld + d;
     T w = hpsi_element<T>(sv, sval, sU, hp, X, u, d);
     if (FUSED) {
-      w = fma(-bn, O[o], w);
+      w = fma(-bn, P[o], w);
       const double x = (double)X[o], wd = (double)w;
       sxw = fma(x, wd, sxw);
       sww = fma(wd, wd, sww);
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(kTileThreads) k_hpsi_tile(SectorView sv, HopPa
   for (int i = threadIdx.x; i < kMaxOrb; i += blockDim.x) sU[i] = Prec<T>::U(hp, i);
   const T* X = X0 + run * vstride;
   T* O = O0 + run * vstride;
+  const T* P = FUSED && ls.prev ? (const T*)ls.prev : O;
   const T bn = FUSED ? (T)ls.beta[(int64_t)run * (ls.mstride + 1) + n] : T(0);
   const bool uni = hp.uniform_u != 0;
   const T u0 = Prec<T>::u0(hp);
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(kTileThreads) k_hpsi_tile(SectorView sv, HopPa
         const int64_t o = (ub + r) * sv.ld + d;
         T w = acc[r];
         if (FUSED) {
-          w = fma(-bn, O[o], w);
+          w = fma(-bn, P[o], w);
           const double xd = (double)x.v[r], wd = (double)w;
           sxw = fma(xd, wd, sxw);
           sww = fma(wd, wd, sww);
@@ -388,10 +391,12 @@ struct Acc16<double> {
 // REG: the value is then selected in registers).  Table loads run one chunk of kPre slots ahead
 // of their use (the table has kEllPad zero slots at its end, so the look-ahead needs no bounds
 // check).
-template <typename T, bool REG>
-__global__ void __launch_bounds__(kRowThreads) k_down_rows(SectorView sv, HopParams hp, const T* __restrict__ X0,
-                                                   T* __restrict__ O0, int64_t vstride, const double* __restrict__ beta,
-                                                   int beta_stride, int n_step, const int* __restrict__ active) {
+// PREV: the vector of the -b term (beta) is P0's, else it is the output's old content.
+template <typename T, bool REG, bool PREV>
+__global__ void __launch_bounds__(kRowThreads) k_down_rows(SectorArgs sv, HopParams hp, const T* __restrict__ X0,
+                                                   T* __restrict__ O0, const T* P0, int64_t vstride,
+                                                   const double* __restrict__ beta, int beta_stride, int n_step,
+                                                   const int* __restrict__ active) {
   constexpr int R = Vec<T>::n;
   constexpr int kPre = kEllPad;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -455,6 +460,11 @@ __global__ void __launch_bounds__(kRowThreads) k_down_rows(SectorView sv, HopPar
       p += kPre * dd;
       const uint32_t bd = sv.B_dn[d];
       const T ed = edn[d];
+      [[maybe_unused]] T pv[R];  // v_{n-1}, requested before the hops
+      if constexpr (PREV) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) pv[r] = u0r + r < du ? P0[run * vstride + (u0r + r) * ld + d] : T(0);
+      }
       Acc16<T> acc;
       {
         const typename Vec<T>::t xv = *reinterpret_cast<const typename Vec<T>::t*>(sxb + d * 16);
@@ -495,7 +505,10 @@ __global__ void __launch_bounds__(kRowThreads) k_down_rows(SectorView sv, HopPar
         if (u0r + r >= du) continue;
         const int64_t o = (u0r + r) * ld + d;
         T out = acc.get(r);
-        if (beta) out -= b * O[o];
+        if (PREV)
+          out -= b * pv[r];
+        else if (beta)
+          out -= b * O[o];
         O[o] = out;
       }
     }
@@ -503,7 +516,7 @@ __global__ void __launch_bounds__(kRowThreads) k_down_rows(SectorView sv, HopPar
 }
 
 template <typename T, bool FUSED>
-__global__ void __launch_bounds__(kThreads, 4) k_up_cols(SectorView sv, HopParams hp, const T* __restrict__ X0,
+__global__ void __launch_bounds__(kThreads, 4) k_up_cols(SectorArgs sv, HopParams hp, const T* __restrict__ X0,
                                                       T* __restrict__ O0, int64_t vstride, int rows_per_cta, int n,
                                                       LanczosScalars ls) {
   using RV = typename Vec<T>::t;
@@ -639,18 +652,27 @@ static void launch_two_pass(const SectorView& sv, const HopParams& hp, const T* 
   const double dim = (double)sv.d_up * sv.d_dn;
   const size_t smem = down_rows_smem(sv, sizeof(T) == 8 ? ED_FP64 : ED_FP32);
   const bool reg = hp.nvals <= 4;
-  allow_max_dynamic_smem(k_down_rows<T, true>);
-  allow_max_dynamic_smem(k_down_rows<T, false>);
   const int64_t groups = (sv.d_up + Vec<T>::n - 1) / Vec<T>::n;
   dim3 g1((unsigned)std::min<int64_t>(groups, 152), runs);
   dim3 g2((unsigned)((sv.d_up + kRowsPerCta - 1) / kRowsPerCta), (unsigned)((sv.d_dn + 32 * Vec<T>::n - 1) / (32 * Vec<T>::n)),
           runs);
   // one timed unit per step: both passes (the second launch is counted separately)
   ProfScope ps_(ls ? K_LANCZOS_STEP : K_HPSI, s, (beta ? 3.0 : 2.0) * es * dim * runs);
-  if (reg)
-    k_down_rows<T, true><<<g1, kRowThreads, smem, s>>>(sv, hp, X, O, vstride, beta, beta_stride, n, ls ? ls->active : nullptr);
+  auto rows = [&](auto r, auto prev) {
+    constexpr bool REG = decltype(r)::value, PREV = decltype(prev)::value;
+    allow_max_dynamic_smem(k_down_rows<T, REG, PREV>);
+    k_down_rows<T, REG, PREV><<<g1, kRowThreads, smem, s>>>(sv, hp, X, O, ls ? (const T*)ls->prev : nullptr, vstride, beta,
+                                                            beta_stride, n, ls ? ls->active : nullptr);
+  };
+  const bool prev = ls && ls->prev;
+  if (reg && prev)
+    rows(std::true_type(), std::true_type());
+  else if (reg)
+    rows(std::true_type(), std::false_type());
+  else if (prev)
+    rows(std::false_type(), std::true_type());
   else
-    k_down_rows<T, false><<<g1, kRowThreads, smem, s>>>(sv, hp, X, O, vstride, beta, beta_stride, n, ls ? ls->active : nullptr);
+    rows(std::false_type(), std::false_type());
   ED_CHECK_LAUNCH();
   note_launch();
   if (ls)

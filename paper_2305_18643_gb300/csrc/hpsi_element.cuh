@@ -16,16 +16,16 @@ template <typename T>
 struct Prec;
 template <>
 struct Prec<double> {
-  __device__ static const double* e_up(const SectorView& s) { return s.e_up; }
-  __device__ static const double* e_dn(const SectorView& s) { return s.e_dn; }
+  __device__ static const double* e_up(const SectorArgs& s) { return s.e_up; }
+  __device__ static const double* e_dn(const SectorArgs& s) { return s.e_dn; }
   __device__ static double val(const HopParams& h, int i) { return h.val[i]; }
   __device__ static double U(const HopParams& h, int i) { return h.U[i]; }
   __device__ static double u0(const HopParams& h) { return h.u0; }
 };
 template <>
 struct Prec<float> {
-  __device__ static const float* e_up(const SectorView& s) { return s.e_up32; }
-  __device__ static const float* e_dn(const SectorView& s) { return s.e_dn32; }
+  __device__ static const float* e_up(const SectorArgs& s) { return s.e_up32; }
+  __device__ static const float* e_dn(const SectorArgs& s) { return s.e_dn32; }
   __device__ static float val(const HopParams& h, int i) { return h.valf[i]; }
   __device__ static float U(const HopParams& h, int i) { return h.Uf[i]; }
   __device__ static float u0(const HopParams& h) { return h.u0f; }

@@ -41,11 +41,13 @@ static int vgrid(int64_t n) {
 template <typename T, typename TO>
 __global__ void __launch_bounds__(kVT) k_lanczos_next(T* __restrict__ W0, const T* __restrict__ X0, int64_t d_up, int64_t d_dn,
                                                       int64_t ld, int64_t vstride, int n, LanczosScalars ls,
-                                                      TO* __restrict__ omega, const double* __restrict__ coef) {
+                                                      TO* __restrict__ omega, const double* __restrict__ coef,
+                                                      T* dst) {
   const int run = blockIdx.y;
   if (!ls.active[run]) return;
   T* W = W0 + run * vstride;
   const T* X = X0 + run * vstride;
+  T* V = dst ? dst + run * vstride : W;
   const double a = ls.alpha[(int64_t)run * ls.mstride + n];
   const double b = ls.beta[(int64_t)run * (ls.mstride + 1) + n + 1];
   const double ib = 1.0 / b;
@@ -55,14 +57,14 @@ __global__ void __launch_bounds__(kVT) k_lanczos_next(T* __restrict__ W0, const 
   for_each_element(d_up, d_dn, [&](int64_t u, int64_t d, int64_t idx) {
     int64_t o = u * ld + d;
     const T vt = (W[o] - aT * X[o]) * ibT;
-    W[o] = vt;
+    V[o] = vt;
     if (omega) omega[idx] += cf * (TO)vt;
     });
 }
 
 void launch_lanczos_next(int dtype, void* W, const void* X, int64_t d_up, int64_t d_dn, int64_t ld, int64_t vstride,
                          int runs, int n, const LanczosScalars& ls, void* omega, const double* coef, cudaStream_t s,
-                         int omega_dtype) {
+                         int omega_dtype, void* dst) {
   dim3 g(vgrid(d_up * d_dn), runs);
   const double es = dtype == ED_FP64 ? 8.0 : 4.0;
   if (omega_dtype < 0) omega_dtype = dtype;
@@ -70,13 +72,13 @@ void launch_lanczos_next(int dtype, void* W, const void* X, int64_t d_up, int64_
   ProfScope ps_(K_LANCZOS_NEXT, s, (3.0 * es + (omega ? 2.0 * eo : 0.0)) * (double)(d_up * d_dn) * runs);
   if (dtype == ED_FP64)
     k_lanczos_next<double, double><<<g, kVT, 0, s>>>((double*)W, (const double*)X, d_up, d_dn, ld, vstride, n, ls,
-                                                      (double*)omega, coef);
+                                                      (double*)omega, coef, (double*)dst);
   else if (omega_dtype == ED_FP64)
     k_lanczos_next<float, double><<<g, kVT, 0, s>>>((float*)W, (const float*)X, d_up, d_dn, ld, vstride, n, ls,
-                                                     (double*)omega, coef);
+                                                     (double*)omega, coef, (float*)dst);
   else
     k_lanczos_next<float, float><<<g, kVT, 0, s>>>((float*)W, (const float*)X, d_up, d_dn, ld, vstride, n, ls,
-                                                    (float*)omega, coef);
+                                                    (float*)omega, coef, (float*)dst);
   ED_CHECK_LAUNCH();
 }
 

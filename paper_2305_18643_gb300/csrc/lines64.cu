@@ -57,10 +57,7 @@ struct LineView {
 struct ClassMap {
   uint8_t of[kMaxVals];  // (magnitude << 1) | (the value is negative)
 };
-// Fills the table for 8 consecutive states per thread, in an order chosen against bank
-// conflicts: the 8 lanes that share a 16-byte shared load gather source groups whose index mod 8
-// differs where that is possible (greedy: states with more entries left first, each taking its most
-// frequent residue still free in the slot).
+// Fills the table for 8 consecutive states per thread, ordered against bank conflicts.
 __global__ void k_line_fill(int64_t dim, const int32_t* __restrict__ ptr, const uint32_t* __restrict__ ent, ClassMap cm,
                             int slots, uint32_t* __restrict__ ell, uint8_t* __restrict__ cnt) {
   const int64_t r0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 8;
@@ -78,6 +75,7 @@ __global__ void k_line_fill(int64_t dim, const int32_t* __restrict__ ptr, const 
 
 // Builds the table of one spin.
 static std::unique_ptr<LineTables> build_lines(const SpinTables& t, const ModelHost& m, cudaStream_t s) {
+  PlainAllocScope plain;  // the table is read on any stream
   auto lt = std::make_unique<LineTables>();
   if (t.dim < 2 || t.nnz == 0 || t.zmax > kLineMaxSlots) return lt;
   ClassMap cm = {};
@@ -144,7 +142,8 @@ __device__ __forceinline__ int is_small(double x, int emax) {
 
 template <bool COLS, bool FUSED, int C>
 __global__ void __launch_bounds__(1024, 1) k_lines64(SectorView sv, HopParams hp, LineView lv, const double* __restrict__ X0,
-                                                  double* __restrict__ O0, int64_t vstride, const double* __restrict__ beta,
+                                                  double* __restrict__ O0, const double* P0, int64_t vstride,
+                                                  const double* __restrict__ beta,
                                                   int beta_stride, int n_step, const int* __restrict__ active,
                                                   LanczosScalars ls) {
   extern __shared__ __align__(16) unsigned char ln_smem[];
@@ -170,6 +169,7 @@ __global__ void __launch_bounds__(1024, 1) k_lines64(SectorView sv, HopParams hp
     const bool two = l0 + 1 < NL;
     const double* Xl = COLS ? X + l0 : X + (int64_t)l0 * ld;
     double* Ol = COLS ? O + l0 : O + (int64_t)l0 * ld;
+    const double* Pl = P0 ? P0 + run * vstride + (int64_t)l0 * ld : Ol;  // v_{n-1} (rows)
     const int64_t pstep = COLS ? ld : 1, lstep = COLS ? 1 : ld;
     const bool pair = COLS && two && wide;  // both columns of a position in one 16-byte access
     __syncthreads();
@@ -305,11 +305,12 @@ __global__ void __launch_bounds__(1024, 1) k_lines64(SectorView sv, HopParams hp
           g1 = hpsi_diag<double>(el1 + ei, d1, sU, false, 0.0);
         }
         y0 = fma(g0, __ldg(xg), y0);
-        if (beta) y0 = fma(-b, o[0], y0);
+        const double* pv = Pl + i;
+        if (beta) y0 = fma(-b, pv[0], y0);
         o[0] = y0;
         if (two) {
           y1 = fma(g1, __ldg(xg + lstep), y1);
-          if (beta) y1 = fma(-b, o[lstep], y1);
+          if (beta) y1 = fma(-b, pv[lstep], y1);
           o[lstep] = y1;
         }
       } else if (pair) {
@@ -435,7 +436,7 @@ void launch_lines64(const SectorView& sv, const HopParams& hp, const double* X, 
     constexpr int C = decltype(c)::value;
     allow_max_dynamic_smem(k_lines64<false, false, C>);
     k_lines64<false, false, C><<<dim3(lines_grid(sv.d_dn, sv.d_up), runs), lines_threads(sv.d_dn), lines_smem(sv.d_dn), s>>>(
-        sv, hp, line_view(*sv.tab_dn->lines), X, O, vstride, beta, beta_stride, n, active, LanczosScalars{});
+        sv, hp, line_view(*sv.tab_dn->lines), X, O, ls ? (const double*)ls->prev : nullptr, vstride, beta, beta_stride, n, active, LanczosScalars{});
   });
   ED_CHECK_LAUNCH();
   note_launch();
@@ -446,10 +447,10 @@ void launch_lines64(const SectorView& sv, const HopParams& hp, const double* X, 
     const LineView up = line_view(*sv.tab_up->lines);
     if (ls) {
       allow_max_dynamic_smem(k_lines64<true, true, C>);
-      k_lines64<true, true, C><<<g, threads, lines_smem(sv.d_up), s>>>(sv, hp, up, X, O, vstride, nullptr, 0, n, active, *ls);
+      k_lines64<true, true, C><<<g, threads, lines_smem(sv.d_up), s>>>(sv, hp, up, X, O, nullptr, vstride, nullptr, 0, n, active, *ls);
     } else {
       allow_max_dynamic_smem(k_lines64<true, false, C>);
-      k_lines64<true, false, C><<<g, threads, lines_smem(sv.d_up), s>>>(sv, hp, up, X, O, vstride, nullptr, 0, n, nullptr,
+      k_lines64<true, false, C><<<g, threads, lines_smem(sv.d_up), s>>>(sv, hp, up, X, O, nullptr, vstride, nullptr, 0, n, nullptr,
                                                                          LanczosScalars{});
     }
   });

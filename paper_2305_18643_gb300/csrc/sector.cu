@@ -223,9 +223,16 @@ std::unique_ptr<SpinTables> build_spin_tables(const ModelHost& m, int N, cudaStr
     hp[k] = PairDev{a, b, (uint32_t)m.pair_vidx[k], between};
   }
   int npairs = (int)hp.size();
-  DevBuf<PairDev> dpairs(std::max(npairs, 1));
+  DevBuf<PairDev> dpairs;
+  DevBuf<int32_t> cnt;
+  DevBuf<int> dz;
+  {
+    PoolScope tmp(s);  // scratch of this call, used on s alone
+    dpairs.alloc(std::max(npairs, 1));
+    cnt.alloc(std::max<int64_t>(dim, 1));
+    dz.alloc(1);
+  }
   if (npairs) ED_CUDA(cudaMemcpyAsync(dpairs.p, hp.data(), npairs * sizeof(PairDev), cudaMemcpyHostToDevice, s));
-  DevBuf<int32_t> cnt(std::max<int64_t>(dim, 1));
   if (dim > 0) {
     { ProfScope ps_(K_TABLES, s, 0.0); k_hop_count<<<nblocks(dim, bs), bs, 0, s>>>(dim, t->basis.p, dpairs.p, npairs, cnt.p); }
     ED_CHECK_LAUNCH();
@@ -243,7 +250,6 @@ std::unique_ptr<SpinTables> build_spin_tables(const ModelHost& m, int N, cudaStr
     ED_CHECK_LAUNCH();
   }
   {
-    DevBuf<int> dz(1);
     ED_CUDA(cudaMemsetAsync(dz.p, 0, sizeof(int), s));
     if (dim > 0) {
       { ProfScope ps_(K_TABLES, s, 0.0); k_max_int<<<std::min<unsigned>(nblocks(dim, bs), 1024), bs, 0, s>>>(cnt.p, dim, dz.p); }

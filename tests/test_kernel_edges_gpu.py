@@ -247,3 +247,14 @@ def test_two_pass_ordered_tables(dtype, many, n_up, n_dn):
     ref = O.apply_h(op, x[:, :dd].cpu().double().numpy()).reshape(du, dd)
     assert np.abs(got[:, :dd] - ref).max() <= (1e-12 if dtype == torch.float64 else 2e-5) * np.abs(ref).max()
     assert np.all(got[:, dd:] == 0.0)
+
+
+# Lanczos vectors written straight into their store, in the forced two-pass form, both precisions.
+@pytest.mark.parametrize("precision", [ed.ED_FP64, ed.ED_FP32])
+def test_two_pass_ground_state_store(precision):
+    c = W.random_cluster(np.random.default_rng(8), 10, 0, 5, 4)
+    E = O.ground_state(O.sector_hamiltonian(_model(c), 5, 4))[0]
+    with ed.Cluster(c, seed=5, precision=precision) as cl:
+        ed.ed_set_option(cl.h, ed.ED_OPT_TWO_PASS_MIN_BYTES, 0.0)
+        st, E0, res, _ = cl.ground_state()
+        assert st == ed.ED_OK and res <= 1e-12 and abs(E0 - E) <= 1e-10 * abs(E)
