@@ -177,9 +177,9 @@ ed_status ed_green_stats(const ed_cluster* c, int64_t* total_steps, int* max_ste
  * persistent ground-state kernel, in which every thread block takes the next cluster from a
  * queue, largest first; a persistent continued-fraction kernel, in which blocks take the
  * continued fractions of more than 8,192 states and, once those are gone, every warp takes the
- * smaller ones one at a time; then the evaluation on the grid and the assembly of G.  The block width and the mapping of the
- * block-level H.psi are picked by timing candidates on the first call for a batch shape (then
- * cached). */
+ * smaller ones one at a time; then the evaluation on the grid and the assembly of G.  Batches with sectors of more than
+ * 8,192 states pick the block width and the mapping of the block-level H.psi by timing candidates
+ * on the first call for a batch shape (then cached). */
 ed_status ed_batch_solve(const ed_cluster_desc* descs, int n, int precision, const double* omega, int n_freq,
                          double eta, int axis, int cf_max_levels, double* E0, double* residual, int* status, int* iters,
                          int64_t* gf_steps, double* G_out, int out_is_device);

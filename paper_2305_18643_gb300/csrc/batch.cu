@@ -12,8 +12,9 @@
 //    (cluster, spin, part, pair) from the queue, applies c+ / c to the ground state and runs the
 //    recursion with the convergence check on the frequency grid.
 // 4. Two grid-wide kernels evaluate every continued fraction on the grid and assemble G.
-// Block width and the element-to-thread mapping of the block-level H.psi are picked by an
-// autotuner on the first call for a given batch shape.  No block ever waits on another block.
+// Block width and the element-to-thread mapping of the block-level H.psi are fixed for sectors of
+// at most 8,192 states, else picked by an autotuner on the first call for a given batch shape.  No
+// block ever waits on another block.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

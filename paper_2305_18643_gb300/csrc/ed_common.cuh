@@ -88,12 +88,13 @@ struct AllocStreamScope {
 
 // Memory of one solve (ground state, Green function) of a cluster with a stream of its own: DevBufs come
 // stream-ordered from a pool of the library, one per device, that keeps at most kPoolKeep bytes between
-// calls and returns the rest to the device when a stream is synchronized (and those too when an allocation
-// of the library finds no memory).  cudaMalloc and cudaFree (which
-// waits for the device) took 4 ms of a 55 ms solve and most of a small one.  Only buffers used on the
-// cluster's stream alone may come from it: the sector tables, which ed_hpsi reads on the caller's stream,
-// are allocated under PlainAllocScope.  Nested scopes (the server's lanes) keep the outer one.  Buffers
-// beyond kPoolMaxAlloc stay with cudaMalloc: the pool would hand them back at every synchronization.
+// calls, returns the rest to the device when a stream is synchronized, and all that it holds unused when an
+// allocation of the library finds no memory.  cudaMalloc and cudaFree (which waits for the device) took 4 ms
+// of a 55 ms solve.  Only buffers used on the cluster's stream alone may come from it: the sector tables,
+// which ed_hpsi reads on the caller's stream, are allocated under PlainAllocScope.  Nested scopes (the
+// server's lanes) keep the outer one.  Buffers beyond kPoolMaxAlloc stay with cudaMalloc: the pool would
+// hand them back at every synchronization (4x4 ground state with its 5 GB chunks in the pool: 1.20 s
+// against 1.03 s).
 constexpr size_t kPoolMaxAlloc = size_t(256) << 20;
 constexpr size_t kPoolKeep = size_t(4) << 30;
 extern thread_local cudaMemPool_t g_alloc_pool;
