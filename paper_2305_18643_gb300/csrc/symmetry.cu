@@ -1437,13 +1437,19 @@ static void sym_green(ed_sym& S, const double* omega, int nz, double eta, int ax
                                                         phi[r].p);
       ED_CHECK_LAUNCH();
     }
-    // the runs of every sector, at most kSymMaxRuns together: the rows' own, then the pairs'
+    // the runs of every sector, at most kSymMaxRuns together and no more than have room for their two
+    // vectors in half of the free memory: the rows' own, then the pairs'
     for (auto& sec : sectors) {
       ed_sym* T = sec.second.get();
       if (T->dim == 0) continue;
       SymMultiStart st = {};
       double2* out[kSymMaxRuns];
-      int R = 0;
+      int R = 0, rmax = 1;
+      size_t fr = 0, tot = 0;
+      if (cudaMemGetInfo(&fr, &tot) == cudaSuccess)
+        rmax = (int)std::max<int64_t>(1, std::min<int64_t>(kSymMaxRuns, (int64_t)(fr / 2) / (16 * T->dim)));
+      else
+        cudaGetLastError();
       auto flush = [&]() {
         if (R) sym_cf_multi(*T, R, st, E0, s_eh, zr, zi, nz, tol, out, s);
         R = 0;
@@ -1452,7 +1458,7 @@ static void sym_green(ed_sym& S, const double* omega, int nz, double eta, int ax
         st.a[R] = x;
         st.b[R] = y;
         out[R] = o;
-        if (++R == kSymMaxRuns) flush();
+        if (++R == rmax) flush();
       };
       for (int r = 0; r < nrow; ++r)
         if (tgt[r] == T) add(phi[r].p, nullptr, D.p + (size_t)r * nz);
