@@ -36,10 +36,8 @@ constexpr int kLinePad = 8;        // slots behind a table, for the look-ahead
 constexpr int kLineBits = 56;
 
 // Hops of one spin, slot-major [slot][dim]: (source << 4) | (magnitude << 1) | sign, so that an entry less
-// its low bits is the byte offset of the source's group.  One list for all magnitudes: tables by
-// magnitude and sign need fewer instructions per hop, but their short loops end at different slots in
-// every lane, and the half-empty gathers cost more shared-memory wavefronts than the instructions
-// saved (rows of the 4x4 sector: 6.3 ms with four lists, 5.0 ms with two, LROWS ms with one).
+// its low bits is the byte offset of the source's group.  One list for all magnitudes: the loops of
+// lists by magnitude and sign end at different slots in every lane, which leaves gathers half empty.
 struct LineTables {
   int classes = 0;  // magnitudes; 0: the spin has too many of them or too many hops
   double mag[kLineMaxClasses] = {};
