@@ -714,9 +714,10 @@ __device__ void warp_hx(const BTable& tu, const BTable& td, const T* D, const T*
 // [m0, m) of the coefficients a, b.
 __device__ __forceinline__ double2 cf_advance(CfForward& st, const double* __restrict__ a, const double* __restrict__ b,
                                               int m0, int m, double b0sq, double2 z, double E0, double s) {
+  const int mask = cf_scale_mask(z);
   for (int n = m0; n < m; ++n) {
     st.level(make_double2(s * (a[n] - E0), n == 0 ? -1.0 : b[n] * b[n]), z);
-    if ((n & 7) == 7) st.rescale();
+    if ((n & mask) == mask) st.rescale();
   }
   st.rescale();
   return st.value(b0sq);

@@ -25,6 +25,10 @@ __device__ __forceinline__ double cf_down_scale(double a, double b, double c, do
   return __hiloint2double(min(max((2046 << 20) - m, 1 << 20), 2045 << 20), 0);
 }
 
+// The rescaling after level n runs where (n & mask) is the mask's first or last value: every eight levels,
+// and after each level for |z| beyond 1e30, where eight levels may leave the range of FP64.
+__device__ __forceinline__ int cf_scale_mask(double2 z) { return fabs(z.x) + fabs(z.y) > 1e30 ? 0 : 7; }
+
 // A level as the recurrences read it: x = s (a_n - E0), y = b_{n+1}^2 (backward; 0 behind the last
 // level) or b_n^2 (forward; -1 for level 0, so that A_1 = 1).
 struct CfBackward {
@@ -85,6 +89,7 @@ constexpr int kCfChunk = 128;  // levels staged in shared memory at a time
 __device__ __forceinline__ double2 cf_eval_block(const double* __restrict__ a, const double* __restrict__ b, int m,
                                                  double b0sq, double2 z, double E0, double s, double2* sm, bool use) {
   CfBackward st;
+  const int mask = cf_scale_mask(z);
   for (int hi = m; hi > 0; hi -= kCfChunk) {
     const int lo = hi > kCfChunk ? hi - kCfChunk : 0;
     __syncthreads();
@@ -96,7 +101,7 @@ __device__ __forceinline__ double2 cf_eval_block(const double* __restrict__ a, c
     if (use)
       for (int n = hi - 1; n >= lo; --n) {
         st.level(sm[n - lo], z);
-        if ((n & 7) == 0) st.rescale();
+        if ((n & mask) == 0) st.rescale();
       }
   }
   return m > 0 ? st.value(b0sq) : make_double2(0.0, 0.0);
@@ -105,6 +110,7 @@ __device__ __forceinline__ double2 cf_eval_block(const double* __restrict__ a, c
 // Advances the forward state of z over levels [m0, m).  Same calling rule.
 __device__ __forceinline__ void cf_advance_block(CfForward& st, const double* __restrict__ a, const double* __restrict__ b,
                                                  int m0, int m, double2 z, double E0, double s, double2* sm, bool use) {
+  const int mask = cf_scale_mask(z);
   for (int lo = m0; lo < m; lo += kCfChunk) {
     const int hi = min(m, lo + kCfChunk);
     __syncthreads();
@@ -114,7 +120,7 @@ __device__ __forceinline__ void cf_advance_block(CfForward& st, const double* __
     if (use)
       for (int n = lo; n < hi; ++n) {
         st.level(sm[n - lo], z);
-        if ((n & 7) == 7) st.rescale();
+        if ((n & mask) == mask) st.rescale();
       }
   }
   st.rescale();

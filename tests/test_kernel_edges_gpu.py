@@ -107,6 +107,21 @@ def test_continued_fraction_grid_edges(nz):
     assert np.abs(G[0] - ref).max() <= 1e-8 and np.abs(G[1] - ref).max() <= 1e-8
 
 
+# Frequencies far outside the spectrum, where eight levels of the recurrences leave the range of FP64: G is
+# 1/z there up to (spectrum / |z|), so z G is the unit matrix to the rounding of the norms.
+@pytest.mark.parametrize("z", [1e20, 1e40, -1e60, 1e140])
+@pytest.mark.parametrize("axis", [ed.ED_AXIS_REAL, ed.ED_AXIS_MATSUBARA])
+def test_continued_fraction_far_frequencies(z, axis):
+    c = W.random_cluster(np.random.default_rng(3), 6, 0, 3, 3)
+    zz = z + 0.05j if axis == ed.ED_AXIS_REAL else 1j * z
+    om = np.array([0.5, z])
+    with ed.Cluster(c, seed=5) as cl:
+        G = cl.green(om, 0.05, axis)
+    B = ed.ed_batch_solve([c], omega=om, eta=0.05, axis=axis, seed=5)[4][0]
+    for g in (G[1], B[0][1], B[1][1]):
+        assert np.abs(zz * g - np.eye(6)).max() <= 1e-10
+
+
 # One-pass H.psi: flat index below 192 columns, tiles of 4, 2 and 1 rows with ragged last tiles and
 # column chunks, rows too long for shared memory; padded rows keep their padding.  FP64 within 1e-12
 # and FP32 within 2e-5 of max|y| (the bounds of the parity tests).
