@@ -239,10 +239,6 @@ SectorView ed_cluster::view(int n_up, int n_dn, int64_t ld) {
   v.ent_dn = d.ent.p;
   v.ell_dn = d.ell.p;
   v.zmax_up = u.zmax;
-  v.tab_up = &u;
-  v.tab_dn = &d;
-  v.model = &model;
-  v.tab_stream = stream;
   v.e_up = u.ediag.p;
   v.e_dn = d.ediag.p;
   v.e_up32 = u.ediag32.p;

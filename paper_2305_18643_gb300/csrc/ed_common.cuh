@@ -242,8 +242,6 @@ struct HopParams {
   float u0f;
 };
 
-struct LineTables;  // lines64.cu
-
 // One spin's sector with N particles: basis, two-level rank tables, hopping table, diagonal.
 struct SpinTables {
   int L = 0, N = 0, split = 0;
@@ -257,7 +255,6 @@ struct SpinTables {
   DevBuf<uint32_t> ell;        // [zmax][dim] slot-major copy: ell[k * dim + r] = k-th entry of row r
   DevBuf<double> ediag;        // [dim] sum_a h_aa n_a
   DevBuf<float> ediag32;       // [dim]
-  std::shared_ptr<LineTables> lines;  // hops by magnitude (lines64.cu), built on first use
 };
 
 // Read-only device view of a two-spin sector for the H.psi kernels.  The two-pass kernels take these fields
@@ -281,11 +278,7 @@ struct SectorArgs {
 
 // With what only the host's choices need.
 struct SectorView : SectorArgs {
-  int zmax_up;              // most hops of an up-spin state
-  SpinTables* tab_up;       // the tables themselves, their model and the stream they are built on
-  SpinTables* tab_dn;
-  const ModelHost* model;
-  cudaStream_t tab_stream;
+  int zmax_up;  // most hops of an up-spin state
 };
 
 // Preset maximum of a continued fraction of the batched and served forms when the caller gives
@@ -358,12 +351,6 @@ void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, c
                          int nblk_cap, cudaStream_t s);
 int lanczos_blocks(const SectorView& sv);   // partial-sum slots per run of the fused step
 int two_pass_blocks(const SectorView& sv, int dtype);
-
-// lines64.cu: FP64 products with integer hop sums.
-bool lines64_usable(const SectorView& sv, cudaStream_t s);
-int lines64_blocks(const SectorView& sv);
-void launch_lines64(const SectorView& sv, const HopParams& hp, const double* X, double* O, int64_t vstride, int runs,
-                    const double* beta, int beta_stride, int n, const LanczosScalars* ls, cudaStream_t s);
 
 // small.cu: many Lanczos levels of small sectors in one launch, a thread-block cluster per run.
 struct SmallStore {  // where the vectors v_{n0 + 1}, v_{n0 + 2}, ... are kept too

@@ -778,7 +778,7 @@ static int one_pass_blocks(const SectorView& sv, int dtype) {
 
 int lanczos_blocks(const SectorView& sv) {
   // capacity for every form (the two-pass column kernel has the most blocks on large sectors)
-  return std::max({one_pass_blocks(sv, ED_FP64), one_pass_blocks(sv, ED_FP32), two_pass_blocks(sv, ED_FP64), lines64_blocks(sv)});
+  return std::max({one_pass_blocks(sv, ED_FP64), one_pass_blocks(sv, ED_FP32), two_pass_blocks(sv, ED_FP64)});
 }
 
 void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const void* x, void* y, cudaStream_t s) {
@@ -787,10 +787,6 @@ void launch_hpsi(const SectorView& sv, const HopParams& hp, int dtype, const voi
 
 void launch_hpsi_block(const SectorView& sv, const HopParams& hp, int dtype, const void* X, void* Y, int64_t vstride,
                        int runs, cudaStream_t s) {
-  if (dtype == ED_FP64 && lines64_usable(sv, s)) {
-    launch_lines64(sv, hp, (const double*)X, (double*)Y, vstride, runs, nullptr, 0, 0, nullptr, s);
-    return;
-  }
   const bool two = use_two_pass(sv, dtype, X, Y, vstride);
   if (dtype == ED_FP64) {
     if (two)
@@ -807,11 +803,6 @@ void launch_hpsi_block(const SectorView& sv, const HopParams& hp, int dtype, con
 
 void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, const void* X, void* XP,
                          int64_t vstride, int runs, int n, const LanczosScalars& ls, int nblk_cap, cudaStream_t s) {
-  if (dtype == ED_FP64 && lines64_usable(sv, s)) {
-    if (lines64_blocks(sv) > nblk_cap) throw Error(ED_ERR_INVALID, "partial buffer too small");
-    launch_lines64(sv, hp, (const double*)X, (double*)XP, vstride, runs, ls.beta, ls.mstride + 1, n, &ls, s);
-    return;
-  }
   const bool two = use_two_pass(sv, dtype, X, XP, vstride);
   if ((two ? two_pass_blocks(sv, dtype) : one_pass_blocks(sv, dtype)) > nblk_cap) throw Error(ED_ERR_INVALID, "partial buffer too small");
   if (dtype == ED_FP64) {

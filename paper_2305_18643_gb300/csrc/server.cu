@@ -55,9 +55,7 @@ size_t spin_table_bytes(int L, int N, int npairs) {
   const int split = L / 2;
   const int64_t nnz = (int64_t)npairs * (int64_t)binomial(L - 2, N - 1);
   const int64_t zmax = std::min<int64_t>(npairs, (int64_t)N * (L - N)) + kEllPad;
-  // (then the tables of lines64.cu)
   return (size_t)d * (4 + 4 + 8 + 4) + 4 + (size_t)std::max<int64_t>(nnz, 1) * 4 + (size_t)zmax * d * 4 +
-         (size_t)d * (4 * (std::min<int64_t>(npairs, (int64_t)N * (L - N)) + 8) + 1) +
          ((size_t(1) << split) + (size_t(1) << (L - split))) * 4 + 4096;
 }
 

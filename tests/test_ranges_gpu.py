@@ -1,0 +1,81 @@
+"""The kernels at the ends of what their entry points take, and in the forms that options select."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2305_18643_gb300 import build, ed
+from paper_2305_18643_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def libed():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    build.build()
+    return ed.lib()
+
+
+def _model(c):
+    return O.Model(c["t"], c["U"], c["mu"], c["eps"], c["theta"])
+
+
+def _product(cl, n_up, n_dn, x, ld):
+    """ed_hpsi on an FP64 vector with leading dimension ld."""
+    du, dd = x.shape
+    xd = torch.zeros((du, ld), dtype=torch.float64, device="cuda")
+    xd[:, :dd] = torch.tensor(x, device="cuda")
+    y = torch.zeros_like(xd)
+    ed.ed_hpsi(cl.h, n_up, n_dn, ed.ED_FP64, xd.data_ptr(), y.data_ptr(), ld, torch.cuda.current_stream().cuda_stream)
+    return y[:, :dd].cpu().numpy()
+
+
+# FP64 products are accurate element by element: every y[u, d] is a sum of at most 64 products in FP64, so it is
+# within 64 2^-53 of (|H| |x|)[u, d] (times two for the reference's own rounding), however small it is
+# beside the rest of its row and column.  Vectors: columns at 1e-10 of the others (a column and all that it hops
+# to, so that sums of small operands alone occur), elements over 30 decades, and everything near 1e-290.
+@pytest.mark.parametrize("kind", ["small columns", "thirty decades", "tiny"])
+@pytest.mark.parametrize("n_up,n_dn,padded", [(6, 7, True), (6, 7, False), (5, 8, True), (4, 5, False)])
+def test_fp64_products_element_by_element(kind, n_up, n_dn, padded):
+    rng = np.random.default_rng(n_up)
+    c = dict(W.served_request(rng, sizes=(14,)), n_up=n_up, n_dn=n_dn)
+    op = O.sector_hamiltonian(_model(c), n_up, n_dn)
+    du, dd = op.shape2
+    x = rng.standard_normal((du, dd))
+    if kind == "small columns":
+        for d0 in (0, dd // 2):
+            x[:, np.append(op.K_dn[d0].indices, d0)] *= 1e-10
+    elif kind == "thirty decades":
+        x *= 10.0 ** rng.uniform(-30.0, 0.0, (du, dd))
+    else:
+        x *= 1e-290
+    with ed.Cluster(c) as cl:
+        got = _product(cl, n_up, n_dn, x, (dd + 127) // 128 * 128 if padded else dd)
+    bound = abs(op.K_up) @ abs(x) + (abs(op.K_dn) @ abs(x).T).T + abs(op.V) * abs(x)
+    assert np.all(np.abs(got - O.apply_h(op, x)) <= 2 * 64 * 2.0 ** -53 * bound)
+
+
+def _launches(fn):
+    n = ed.ed_launch_count()
+    fn()
+    return ed.ed_launch_count() - n
+
+
+# ED_OPT_TWO_PASS_MIN_BYTES selects the form of every product: two launches with 0, one beyond every size.
+@pytest.mark.parametrize("dtype", [ed.ED_FP64, ed.ED_FP32])
+@pytest.mark.parametrize("L,n_up,n_dn", [(8, 4, 4), (13, 6, 7)])
+def test_two_pass_option_selects_the_product(L, n_up, n_dn, dtype):
+    c = dict(W.served_request(np.random.default_rng(1), sizes=(8,)) if L == 8 else
+             W.random_cluster(np.random.default_rng(1), L, 0, n_up, n_dn, U=4.0), n_up=n_up, n_dn=n_dn)
+    with ed.Cluster(c) as cl:
+        du, dd = ed.ed_sector_dims(cl.h, n_up, n_dn)
+        ld = (dd + 127) // 128 * 128
+        x = torch.zeros((du, ld), dtype=torch.float64 if dtype == ed.ED_FP64 else torch.float32, device="cuda")
+        y = torch.zeros_like(x)
+        for value, launches in ((0.0, 2), (9.1e18, 1)):
+            ed.ed_set_option(cl.h, ed.ED_OPT_TWO_PASS_MIN_BYTES, value)
+            assert _launches(lambda: ed.ed_hpsi(cl.h, n_up, n_dn, dtype, x.data_ptr(), y.data_ptr(), ld,
+                                                torch.cuda.current_stream().cuda_stream)) == launches
