@@ -575,6 +575,13 @@ __device__ void block_ground_state(BCluster& c, const BTable* tabs, GSShared& g,
     bred3(r2, q1, q2, g.bs);
     res = sqrt(fmax(r2, 0.0));
     const double scale = fmax(1.0, fabs(E));
+    // the second eigenvalue, where a comparison below hangs on its last digits
+    const double off = g.eval[3], g32 = fp64 ? 0.0 : res * res / (1e-11 * scale);
+    if (fabs(lam1 - lam0 - degenerate_gap(lam0)) <= off || (!fp64 && (fabs(lam1 - E) <= off || fabs(lam1 - E - g32) <= off))) {
+      tridiag_second_block(g.alpha, g.beta, m, g.eval, g.svec + m);
+      __syncthreads();
+      lam1 = g.eval[1];
+    }
     if (fp64 || c.precision == ED_FP64)
       ok = res / scale <= c.tol || brk;
     else
@@ -587,7 +594,7 @@ __device__ void block_ground_state(BCluster& c, const BTable* tabs, GSShared& g,
     c.residual = res / fmax(1.0, fabs(E));
     c.iters = total;
     c.gap = lam1 - lam0;
-    c.status = !ok ? ED_WARN_NOT_CONVERGED : ((lam1 - lam0) < 1e-8 * fmax(1.0, fabs(lam0)) ? ED_WARN_DEGENERATE : ED_OK);
+    c.status = !ok ? ED_WARN_NOT_CONVERGED : (lam1 - lam0 < degenerate_gap(lam0) ? ED_WARN_DEGENERATE : ED_OK);
   }
   __syncthreads();
 }

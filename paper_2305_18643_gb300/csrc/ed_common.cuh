@@ -378,8 +378,12 @@ void launch_axpby(int dtype_y, void* y, int dtype_a, const void* a, const double
 // y[u][d] (leading dimension ld_y) = scale * a[u][d] (leading dimension ld_a); scale NULL = 1.
 void launch_copy_ld(int dty, void* y, int64_t ld_y, int dta, const void* a, int64_t ld_a, const double* scale,
                     int64_t d_up, int64_t d_dn, cudaStream_t s);
+void launch_tridiag_second(const double* alpha, const double* beta, int n, double* out_eval, double* scratch, cudaStream_t s);
 void launch_tridiag_lowest(const double* alpha, const double* beta, int n, double* out_eval,
                            double* out_vec, cudaStream_t s);
+
+// Gaps below this above a ground energy E0 raise ED_WARN_DEGENERATE.
+__host__ __device__ inline double degenerate_gap(double E0) { return 1e-8 * fmax(1.0, fabs(E0)); }
 
 struct GroundResult {
   double E0 = 0, residual = 0, gap = 0;

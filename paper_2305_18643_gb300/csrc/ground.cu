@@ -296,11 +296,17 @@ static int lanczos_pass(ed_cluster& c, const SectorView& sv, int dtype, LanczosR
           *breakdown = levels < L.M;
         }
         launch_tridiag_lowest(L.alpha.p, L.beta.p, levels, L.evals.p, L.svec.p, s);
-        ED_CUDA(cudaMemcpyAsync(host, L.evals.p, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        ED_CUDA(cudaMemcpyAsync(host, L.evals.p, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
         ED_CUDA(cudaStreamSynchronize(s));
         m = levels;
         if (!act || host[2] < tol_ritz * std::max(1.0, std::fabs(host[0]))) break;
       }
+    }
+    // the second eigenvalue, where the caller's comparison hangs on its last digits
+    if (pass == 0 && std::fabs(host[1] - host[0] - degenerate_gap(host[0])) <= host[3]) {
+      launch_tridiag_second(L.alpha.p, L.beta.p, m, L.evals.p, L.svec.p + m, s);
+      ED_CUDA(cudaMemcpyAsync(host + 1, L.evals.p + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
+      ED_CUDA(cudaStreamSynchronize(s));
     }
     if (pass == 0 && store.ok && store.count >= m) {
       ritz_sum(dtype, store, 0, m, L.svec.p, omega64, du, dd, ld, 0, s);
@@ -509,7 +515,7 @@ GroundResult run_ground_state(ed_cluster& c, int dtype, double tol, int max_iter
     R.residual = res_abs / scale;
     R.iters = total_iters;
     R.gap = lam1 - lam0;
-    R.degenerate = (lam1 - lam0) < 1e-8 * std::max(1.0, std::fabs(lam0));
+    R.degenerate = lam1 - lam0 < degenerate_gap(lam0);
     if (ok) {
       R.converged = true;
       break;

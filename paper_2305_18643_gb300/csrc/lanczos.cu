@@ -222,6 +222,17 @@ __global__ void __launch_bounds__(kVT) k_tridiag_lowest(const double* __restrict
   for (int i = threadIdx.x; i < n; i += blockDim.x) vec[i] = sv[i];
 }
 
+__global__ void __launch_bounds__(kVT) k_tridiag_second(const double* __restrict__ a, const double* __restrict__ b, int n,
+                                                        double* __restrict__ out_eval, double* __restrict__ scratch) {
+  tridiag_second_block(a, b, n, out_eval, scratch);
+}
+
+void launch_tridiag_second(const double* alpha, const double* beta, int n, double* out_eval, double* scratch, cudaStream_t s) {
+  ProfScope ps_(K_TRIDIAG, s, 0.0);
+  k_tridiag_second<<<1, kVT, 0, s>>>(alpha, beta, n, out_eval, scratch);
+  ED_CHECK_LAUNCH();
+}
+
 void launch_tridiag_lowest(const double* alpha, const double* beta, int n, double* out_eval, double* out_vec,
                            cudaStream_t s) {
   const size_t smem = (4 * (size_t)n + 1) * sizeof(double);

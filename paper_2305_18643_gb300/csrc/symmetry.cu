@@ -871,7 +871,7 @@ static void sym_ground_state(ed_sym& S, double tol, int max_iter, uint64_t seed)
   const int M = std::max(2, (int)std::min<int64_t>(max_iter > 0 ? max_iter : 600, dim));
   const int nb = sym_grid(dim, kSymRowsPerBlock), nv = sym_grid(vlen, kSymThreads * 4);
   const int np = std::max(nb, nv);
-  DevBuf<double> V0(vlen), V1(vlen), W(vlen), start(vlen), alpha(M + 1), beta(M + 2), evals(3), svec(2 * (M + 2)), part(np),
+  DevBuf<double> V0(vlen), V1(vlen), W(vlen), start(vlen), alpha(M + 1), beta(M + 2), evals(4), svec(2 * (M + 2)), part(np),
       part2(np);
   DevBuf<unsigned> tk(2);
   ED_CUDA(cudaMemsetAsync(tk.p, 0, 2 * sizeof(unsigned), s));

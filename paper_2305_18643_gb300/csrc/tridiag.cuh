@@ -9,8 +9,8 @@
 // runs only where it decides something: both eigenvalues are first located to a few ulps of the
 // matrix norm with the division-free recurrence p_k = (a_k - x) p_{k-1} - b_k^2 p_{k-2} on entries scaled
 // by a power of two (three rounds in FP32 on every thread, then FP64 on 16 lanes per eigenvalue);
-// the multisection for the lowest one then counts only at points inside that uncertainty, and
-// its result is bit for bit that of counting at every point.
+// the multisection then counts only at points inside that uncertainty, and its result is bit for bit that
+// of counting at every point.
 //
 // One call, over the checks of a 100-level run: 927 us with the quotient form at every point and a
 // division per pivot and sweep, 254 us now; over those of a 160-level run 1,418 and 380 us.  The ground
@@ -77,17 +77,12 @@ static __device__ inline int sturm_count(const double* __restrict__ a, const dou
   return cnt;
 }
 
-// out_eval: [0] lowest eigenvalue, [1] second eigenvalue (inf if n < 2), [2] Ritz estimate
-// b_n |s_{n-1}|.  vec: [0, n) unit eigenvector of the lowest eigenvalue (s_0 >= 0), [n, 2n) scratch.
-// The block has a multiple of 32 threads, at least 64.
-static __device__ void tridiag_lowest_block(const double* __restrict__ a, const double* __restrict__ b, int n,
-                                            double* out_eval, double* vec) {
+// Gershgorin interval [lo, hi] of the matrix, padded.  All threads of the block must call it.
+static __device__ __forceinline__ void tridiag_interval(const double* __restrict__ a, const double* __restrict__ b, int n, double* out_lo,
+                                               double* out_hi) {
   __shared__ double s_lo, s_hi;
-  __shared__ int s_first[2];
-  __shared__ double s_near[2], s_width;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-  // Gershgorin interval
-  if (tid < 32) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
     double lo = 1e300, hi = -1e300;
     for (int i = lane; i < n; i += 32) {
       const double r = (i > 0 ? fabs(b[i]) : 0.0) + (i + 1 < n ? fabs(b[i + 1]) : 0.0);
@@ -105,7 +100,68 @@ static __device__ void tridiag_lowest_block(const double* __restrict__ a, const 
     }
   }
   __syncthreads();
-  const double glo = s_lo, ghi = s_hi;
+  *out_lo = s_lo;
+  *out_hi = s_hi;
+}
+
+// Multisection of [lo, hi] for the k-th lowest eigenvalue (from 1) with blockDim.x points a round, given
+// that it lies within `slack` of `near` for any matrix within rounding of this one: points further away
+// need no count, and points that round to the same number need one.  cand: room for ncand ints.  All
+// threads of the block must call it; the midpoint of the last interval is returned to each.
+static __device__ __forceinline__ double tridiag_multisect(const double* __restrict__ a, const double* __restrict__ b, int n, int k, double lo,
+                                                  double hi, double near, double slack, int* cand, int ncand) {
+  __shared__ int s_first, s_cand;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  auto point = [&](int j) { return lo + (hi - lo) * (double)(j + 1) / (double)(nt + 1); };
+  for (int round = 0; round < 16; ++round) {
+    if (tid == 0) {
+      s_first = nt;
+      s_cand = 0;
+    }
+    __syncthreads();
+    const double x = point(tid);
+    if (x > near + slack) {
+      atomicMin(&s_first, tid);
+    } else if (x >= near - slack && (tid == 0 || point(tid - 1) != x)) {
+      const int c = atomicAdd(&s_cand, 1);
+      if (c < ncand) cand[c] = tid;
+    }
+    __syncthreads();
+    const int nc = s_cand;
+    if (nc <= ncand) {
+      for (int c = tid; c < nc; c += nt) {
+        const int j = cand[c];
+        if (sturm_count(a, b, n, point(j)) >= k) atomicMin(&s_first, j);
+      }
+    } else if (x >= near - slack && x <= near + slack) {
+      if (sturm_count(a, b, n, x) >= k) atomicMin(&s_first, tid);
+    }
+    __syncthreads();
+    const int j = s_first;
+    const double nlo = j == 0 ? lo : lo + (hi - lo) * (double)j / (double)(nt + 1);
+    const double nhi = j == nt ? hi : lo + (hi - lo) * (double)(j + 1) / (double)(nt + 1);
+    lo = nlo;
+    hi = nhi;
+    __syncthreads();
+    if (hi - lo <= 4e-16 * fmax(fabs(lo), fabs(hi))) break;
+  }
+  return 0.5 * (lo + hi);
+}
+
+// How far the brackets of the division-free counts may be off: their width and 100 ulps of the norm (both
+// counts are exact for matrices within ~10 ulps of this one).
+static __device__ __forceinline__ double tridiag_slack(double width, double sc) { return 0.5 * width + 100.0 * 2.3e-16 * sc; }
+
+// out_eval: [0] lowest eigenvalue, [1] about the second eigenvalue (inf if n < 2; tridiag_second_block
+// settles it), [2] Ritz estimate b_n |s_{n-1}|, [3] how far [1] may be off.  vec: [0, n) unit eigenvector of the lowest eigenvalue (s_0 >= 0), [n, 2n) scratch.
+// The block has a multiple of 32 threads, at least 64.
+static __device__ void tridiag_lowest_block(const double* __restrict__ a, const double* __restrict__ b, int n,
+                                            double* out_eval, double* vec) {
+  __shared__ int s_first[2];
+  __shared__ double s_near[2], s_width[2];
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  double glo, ghi;
+  tridiag_interval(a, b, n, &glo, &ghi);
   // scale by a power of two (exact), so that |entries|, |x| <= 1/2 and |a - x| <= 1
   int ex;
   frexp(fmax(fabs(glo), fabs(ghi)), &ex);
@@ -176,51 +232,15 @@ static __device__ void tridiag_lowest_block(const double* __restrict__ a, const 
       }
       if (__all_sync(0xffffffffu, done)) break;
     }
-    if (pt == 0) s_near[e] = 0.5 * (dlo + dhi) * sc;
-    if (lane == 0) s_width = (dhi - dlo) * sc;
+    if (pt == 0) {
+      s_near[e] = 0.5 * (dlo + dhi) * sc;
+      s_width[e] = (dhi - dlo) * sc;
+    }
   }
   __syncthreads();
-  // multisection for the lowest eigenvalue on nt points a round; both counts are exact for matrices
-  // within ~10 ulps (of the norm) of this one, so points further than 100 ulps from the bracket need
-  // none, and points that round to the same number need one
-  const double near = s_near[0], slack = 0.5 * s_width + 100.0 * 2.3e-16 * sc;
-  int* cand = reinterpret_cast<int*>(vec);
-  double rlo = glo, rhi = ghi;
-  auto point = [&](int j) { return rlo + (rhi - rlo) * (double)(j + 1) / (double)(nt + 1); };
-  for (int round = 0; round < 16; ++round) {
-    if (tid == 0) {
-      s_first[0] = nt;
-      s_first[1] = 0;
-    }
-    __syncthreads();
-    const double x = point(tid);
-    if (x > near + slack) {
-      atomicMin(&s_first[0], tid);
-    } else if (x >= near - slack && (tid == 0 || point(tid - 1) != x)) {
-      const int c = atomicAdd(&s_first[1], 1);
-      if (c < 4 * n) cand[c] = tid;  // vec holds 2 n doubles
-    }
-    __syncthreads();
-    const int nc = s_first[1];
-    if (nc <= 4 * n) {
-      for (int c = tid; c < nc; c += nt) {
-        const int j = cand[c];
-        if (sturm_count(a, b, n, point(j)) >= 1) atomicMin(&s_first[0], j);
-      }
-    } else if (x >= near - slack && x <= near + slack) {
-      if (sturm_count(a, b, n, x) >= 1) atomicMin(&s_first[0], tid);
-    }
-    __syncthreads();
-    const int j = s_first[0];
-    const double nlo = j == 0 ? rlo : rlo + (rhi - rlo) * (double)j / (double)(nt + 1);
-    const double nhi = j == nt ? rhi : rlo + (rhi - rlo) * (double)(j + 1) / (double)(nt + 1);
-    rlo = nlo;
-    rhi = nhi;
-    __syncthreads();
-    if (rhi - rlo <= 4e-16 * fmax(fabs(rlo), fabs(rhi))) break;
-  }
+  const double lam = tridiag_multisect(a, b, n, 1, glo, ghi, s_near[0], tridiag_slack(s_width[0], sc), reinterpret_cast<int*>(vec),
+                                       4 * n);  // vec holds 2 n doubles
   if (tid >= 32) return;
-  const double lam = 0.5 * (rlo + rhi);
   // inverse iteration with shift just below lam: T - sigma I is positive definite, so the
   // Thomas elimination without pivoting is stable.  The pivots m_i are those of every iteration, so
   // they are found once (lane 0; cp_i = b_{i+1} / m_i is kept); the quotients by m_i in the sweeps
@@ -280,7 +300,21 @@ static __device__ void tridiag_lowest_block(const double* __restrict__ a, const 
     out_eval[0] = lam;
     out_eval[1] = n < 2 ? INFINITY : s_near[1];
     out_eval[2] = fabs(b[n]) * fabs(y[n - 1]);
+    out_eval[3] = tridiag_slack(s_width[1], sc);
   }
+}
+
+// The second eigenvalue by counts of record, bit for bit that of counting at every point, from what
+// tridiag_lowest_block left in out_eval for the same matrix.  Callers compare gaps with thresholds, and need it
+// only where a threshold lies within out_eval[3] of theirs: in every check it made the ground states of 64
+// clusters of at most 6 orbitals 13 % slower, after every run those of a 2x4 cluster 5 %.  scratch: n doubles.
+static __device__ void tridiag_second_block(const double* __restrict__ a, const double* __restrict__ b, int n, double* out_eval,
+                                            double* scratch) {
+  if (n < 2) return;
+  double glo, ghi;
+  tridiag_interval(a, b, n, &glo, &ghi);
+  const double lam = tridiag_multisect(a, b, n, 2, glo, ghi, out_eval[1], out_eval[3], reinterpret_cast<int*>(scratch), 2 * n);
+  if (threadIdx.x == 0) out_eval[1] = lam;
 }
 
 }  // namespace ed

@@ -1,5 +1,9 @@
 """The kernels at the ends of what their entry points take, and in the forms that options select."""
 
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -79,3 +83,38 @@ def test_two_pass_option_selects_the_product(L, n_up, n_dn, dtype):
             ed.ed_set_option(cl.h, ed.ED_OPT_TWO_PASS_MIN_BYTES, value)
             assert _launches(lambda: ed.ed_hpsi(cl.h, n_up, n_dn, dtype, x.data_ptr(), y.data_ptr(), ld,
                                                 torch.cuda.current_stream().cuda_stream)) == launches
+
+
+@pytest.fixture(scope="module")
+def tridiag(tmp_path_factory):
+    here = os.path.dirname(os.path.abspath(__file__))
+    so = str(tmp_path_factory.mktemp("tridiag") / "tridiag_reference.so")
+    subprocess.run([build.nvcc()] + build.ARCH + build.FLAGS + ["-shared", "-o", so, os.path.join(here, "tridiag_reference.cu")],
+                   check=True)
+    return ctypes.CDLL(so)
+
+
+# Both eigenvalues, the eigenvector and the Ritz estimate bit for bit those of the plain form: random Lanczos
+# coefficients, a chain broken into equal halves (a double lowest eigenvalue), a diagonal matrix, and Wilkinson's
+# matrix (pairs of eigenvalues close together).
+@pytest.mark.parametrize("kind", ["random", "halves", "diagonal", "wilkinson"])
+@pytest.mark.parametrize("n", [1, 2, 3, 33, 600])
+@pytest.mark.parametrize("threads", [64, 256])
+def test_tridiagonal_bit_for_bit(tridiag, kind, n, threads):
+    rng = np.random.default_rng(n)
+    a, b = rng.standard_normal(n) - 3.0, rng.uniform(0.1, 3.0, n + 1)
+    if kind == "halves":
+        a[n // 2:n // 2 * 2], b[n // 2 + 1:n // 2 * 2] = a[:n // 2], b[1:n // 2]
+        b[n // 2] = 0.0
+    elif kind == "diagonal":
+        b[:] = 0.0
+    elif kind == "wilkinson":
+        a, b = np.abs(np.arange(n) - (n - 1) / 2.0), np.ones(n + 1)
+    for scale in (1e-7, 1.0, 1e6):
+        ab = [torch.tensor(v * scale, device="cuda") for v in (a, b)]
+        out = [torch.zeros(m, dtype=torch.float64, device="cuda") for m in (4, 2 * n, 4, 2 * n)]
+        assert tridiag.tridiag_both(*[ctypes.c_void_p(t.data_ptr()) for t in ab], n, threads,
+                                    *[ctypes.c_void_p(t.data_ptr()) for t in out]) == 0
+        fast, vec, plain, ref = [t.cpu().numpy() for t in out]
+        assert np.array_equal(fast[:3], plain[:3])
+        assert np.array_equal(vec[:n], ref[:n])
