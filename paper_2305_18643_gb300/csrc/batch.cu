@@ -723,8 +723,11 @@ __device__ __forceinline__ double2 cf_advance(CfForward& st, const double* __res
                                               int m0, int m, double b0sq, double2 z, double E0, double s) {
   const int mask = cf_scale_mask(z);
   for (int n = m0; n < m; ++n) {
-    st.level(make_double2(s * (a[n] - E0), n == 0 ? -1.0 : b[n] * b[n]), z);
-    if ((n & mask) == mask) st.rescale();
+    const double2 e = make_double2(s * (a[n] - E0), n == 0 ? -1.0 : b[n] * b[n]);
+    const bool wide = cf_wide(e);
+    if (wide) st.rescale();
+    st.level(e, z);
+    if (wide || (n & mask) == mask) st.rescale();
   }
   st.rescale();
   return st.value(b0sq);

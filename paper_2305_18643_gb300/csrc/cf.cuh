@@ -26,8 +26,14 @@ __device__ __forceinline__ double cf_down_scale(double a, double b, double c, do
 }
 
 // The rescaling after level n runs where (n & mask) is the mask's first or last value: every eight levels,
-// and after each level for |z| beyond 1e30, where eight levels may leave the range of FP64.
+// and after each level for |z| beyond 1e30, where eight levels may leave the range of FP64.  A level whose own
+// coefficients are that large (cf_wide) is rescaled before and after.
 __device__ __forceinline__ int cf_scale_mask(double2 z) { return fabs(z.x) + fabs(z.y) > 1e30 ? 0 : 7; }
+
+// |x| of a level beyond 2^100 or its y beyond 2^200 (by the exponents: no FP64 comparison).
+__device__ __forceinline__ bool cf_wide(double2 e) {
+  return (__double2hiint(e.x) & 0x7fffffff) > ((1023 + 100) << 20) || __double2hiint(e.y) > ((1023 + 200) << 20);
+}
 
 // A level as the recurrences read it: x = s (a_n - E0), y = b_{n+1}^2 (backward; 0 behind the last
 // level) or b_n^2 (forward; -1 for level 0, so that A_1 = 1).
@@ -100,8 +106,11 @@ __device__ __forceinline__ double2 cf_eval_block(const double* __restrict__ a, c
     __syncthreads();
     if (use)
       for (int n = hi - 1; n >= lo; --n) {
-        st.level(sm[n - lo], z);
-        if ((n & mask) == 0) st.rescale();
+        const double2 e = sm[n - lo];
+        const bool wide = cf_wide(e);
+        if (wide) st.rescale();
+        st.level(e, z);
+        if (wide || (n & mask) == 0) st.rescale();
       }
   }
   return m > 0 ? st.value(b0sq) : make_double2(0.0, 0.0);
@@ -119,8 +128,11 @@ __device__ __forceinline__ void cf_advance_block(CfForward& st, const double* __
     __syncthreads();
     if (use)
       for (int n = lo; n < hi; ++n) {
-        st.level(sm[n - lo], z);
-        if ((n & mask) == mask) st.rescale();
+        const double2 e = sm[n - lo];
+        const bool wide = cf_wide(e);
+        if (wide) st.rescale();
+        st.level(e, z);
+        if (wide || (n & mask) == mask) st.rescale();
       }
   }
   st.rescale();

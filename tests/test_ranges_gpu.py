@@ -85,6 +85,21 @@ def test_two_pass_option_selects_the_product(L, n_up, n_dn, dtype):
                                                 torch.cuda.current_stream().cuda_stream)) == launches
 
 
+# Continued fractions of clusters whose energies are far beyond the frequencies: eight levels of the recurrences leave
+# the range of FP64 by the coefficients alone.  Within 1e-8 of the largest |G| of the exact Lehmann sum.
+@pytest.mark.parametrize("scale", [2.0 ** 40, 2.0 ** 130, 2.0 ** 200])
+def test_continued_fraction_huge_energies(scale):
+    c = W.random_cluster(np.random.default_rng(3), 6, 0, 3, 3)
+    om = np.array([0.0, 0.5, -2.0])
+    ref = O.green_exact(_model(c), 3, 3, (om + 0.05j) / scale)[0] / scale
+    c = dict(c, t=c["t"] * scale, U=c["U"] * scale, mu=c["mu"] * scale)
+    with ed.Cluster(c, seed=5) as cl:
+        G = cl.green(om, 0.05)
+    B = ed.ed_batch_solve([c], omega=om, eta=0.05, seed=5)[4][0]
+    for g in (G, B[0], B[1]):
+        assert np.abs(g - ref).max() <= 1e-8 * np.abs(ref).max()
+
+
 @pytest.fixture(scope="module")
 def tridiag(tmp_path_factory):
     here = os.path.dirname(os.path.abspath(__file__))
