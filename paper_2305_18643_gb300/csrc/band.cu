@@ -387,6 +387,9 @@ __global__ void __launch_bounds__(kSvqbThreads) k_svqb(const double* __restrict_
     tot = s_tot[0] + s_tot[1] + s_tot[2] + s_tot[3];
     __syncthreads();
     if (!(off > 1e-26 * tot)) break;
+    int ex;
+    frexp(tot, &ex);
+    const double unit = ldexp(1.0, -(ex >> 1));  // brings the entries to 1 for the FP32 quotients
     for (int round = 0; round < m - 1; ++round) {
       if (tid < half) {  // pair tid: positions tid and m - 1 - tid of the round-robin circle
         const int pa = tid, pb = m - 1 - tid;
@@ -399,9 +402,9 @@ __global__ void __launch_bounds__(kSvqbThreads) k_svqb(const double* __restrict_
         }
         double c = 1.0, s = 0.0;
         if (q < p) {
-          const float arq = (float)a[r][q];
+          const float arq = (float)(unit * a[r][q]);
           if (arq != 0.f) {
-            const float theta = (float)(a[q][q] - a[r][r]) / (2.f * arq);
+            const float theta = (float)(unit * (a[q][q] - a[r][r])) / (2.f * arq);
             const double t = (double)((theta >= 0.f ? 1.f : -1.f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f))));
             c = rsqrt(fma(t, t, 1.0));
             s = t * c;

@@ -100,6 +100,20 @@ def test_continued_fraction_huge_energies(scale):
         assert np.abs(g - ref).max() <= 1e-8 * np.abs(ref).max()
 
 
+# Band Lanczos of the same clusters: the Gram matrices hold the squares of the energies, beyond the range of FP32.
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 70, 2.0 ** 200])
+@pytest.mark.parametrize("ns", [3, 8])
+def test_band_huge_energies(scale, ns):
+    c = W.random_cluster(np.random.default_rng(ns), ns, 0, 2, 1)
+    om = W.matsubara_grid(17) * scale
+    ref = O.green_exact(_model(c), 2, 1, 1j * om / scale)[0] / scale
+    c = dict(c, t=c["t"] * scale, U=c["U"] * scale, mu=c["mu"] * scale)
+    with ed.Cluster(c, seed=5, gf_method=ed.ED_GF_BAND) as cl:
+        ed.ed_set_option(cl.h, ed.ED_OPT_GF_TOL, 1e-10 / scale)  # an absolute change of G
+        G = cl.green(om, 0.0, axis=ed.ED_AXIS_MATSUBARA)
+    assert np.abs(G - ref).max() <= 1e-8 * np.abs(ref).max()
+
+
 @pytest.fixture(scope="module")
 def tridiag(tmp_path_factory):
     here = os.path.dirname(os.path.abspath(__file__))
