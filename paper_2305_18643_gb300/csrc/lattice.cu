@@ -49,8 +49,8 @@ __device__ __forceinline__ double2 shfl2(double2 v, int src, int width) {
 // whose entry in column k has the largest max(|re|, |im|) (within sqrt(2) of the largest modulus;
 // compared as integers, off the FP64 pipe).  The rows rotate through the registers, so that the
 // pivot row is always c[0] and every register index is static.  On return lane j holds column `dst`
-// of the inverse (row swaps become column swaps).  Returns false if a pivot is zero or NaN.  All
-// lanes of the warp must call it.
+// of the inverse (row swaps become column swaps).  Returns false if the squared modulus of a pivot is
+// zero (its reciprocal is taken from it, so below ~1e-162 too) or NaN.  All lanes of the warp must call it.
 template <int M>
 __device__ __forceinline__ bool group_invert(double2 (&c)[M], int L, int& dst) {
   const int j = threadIdx.x & (M - 1);
@@ -72,8 +72,6 @@ __device__ __forceinline__ bool group_invert(double2 (&c)[M], int L, int& dst) {
       }
     }
     p = __shfl_sync(0xffffffffu, p, k, M);
-    best = __shfl_sync(0xffffffffu, best, k, M);
-    if (best == 0ull || best > (0x7ff0000000000000ull << 1)) ok = false;
     if (j == k) prow = k + p;
     // swaps by selects on values (a branch on i == p would index the registers)
     const double2 top = c[0];
@@ -85,7 +83,9 @@ __device__ __forceinline__ bool group_invert(double2 (&c)[M], int L, int& dst) {
       r = make_double2(h ? v.x : r.x, h ? v.y : r.y);
       c[i] = make_double2(h ? top.x : v.x, h ? top.y : v.y);
     }
-    const double2 inv = cinv(shfl2(r, k, M));
+    const double2 pivot = shfl2(r, k, M);
+    if (!(cabs2(pivot) > 0.0)) ok = false;
+    const double2 inv = cinv(pivot);
     const double2 f0 = j == k ? inv : cmul(r, inv);  // the scaled pivot row
 #pragma unroll
     for (int i = 1; i < M; ++i) {

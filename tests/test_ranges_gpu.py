@@ -114,6 +114,15 @@ def test_band_huge_energies(scale, ns):
     assert np.abs(G - ref).max() <= 1e-8 * np.abs(ref).max()
 
 
+# Matrices whose pivots' squares underflow are refused, not answered with infinities.
+@pytest.mark.parametrize("L", [1, 2, 5, 17])
+def test_cpt_refuses_underflowing_pivots(L):
+    lat = W.square_superlattice(L, 1, -0.1)
+    Gc = np.tile((np.eye(L) + 0.1j) * 1e-170, (3, 1, 1))
+    with pytest.raises(ed.EDError):
+        ed.ed_cpt_green(lat, Gc, np.zeros((1, 1)))
+
+
 @pytest.fixture(scope="module")
 def tridiag(tmp_path_factory):
     here = os.path.dirname(os.path.abspath(__file__))
