@@ -159,14 +159,16 @@ __global__ void k_build_v(const double* __restrict__ kt, int nk, int D, const in
   }
 }
 
-// ph[k][R] = e^{-i k.r_R}, the phases of the periodization (Eq. CPT3).
+// ph[k][R] = e^{-i k.(r_R - r_0)}, the phases of the periodization (Eq. CPT3).  Only products of one with the
+// conjugate of another are used, and from the first site the phases are as small as the cluster, wherever
+// its origin lies.
 __global__ void k_site_phases(const double* __restrict__ kt, const double* __restrict__ pos, int D, int L, int nk,
                               double2* __restrict__ ph) {
   const int64_t n = (int64_t)nk * L;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const int k = (int)(t / L), r = (int)(t % L);
     double x = 0.0;
-    for (int d = 0; d < D; ++d) x += kt[k * D + d] * pos[r * D + d];
+    for (int d = 0; d < D; ++d) x += kt[k * D + d] * (pos[r * D + d] - pos[d]);
     double sn, cs;
     sincos(-x, &sn, &cs);
     ph[t] = make_double2(cs, sn);

@@ -123,6 +123,18 @@ def test_cpt_refuses_underflowing_pivots(L):
         ed.ed_cpt_green(lat, Gc, np.zeros((1, 1)))
 
 
+# The periodized G depends on differences of site positions alone: an origin at 2^33 lattice constants (where the
+# positions are still exact) changes nothing.
+def test_periodized_cpt_far_origin():
+    rng = np.random.default_rng(2)
+    lat = W.square_superlattice(2, 2, -1.0, 0.3)
+    kt = rng.uniform(-3, 3, (9, 2))
+    Gc = np.linalg.inv((2.0 + 1.0j) * np.eye(4) + 0.1 * rng.standard_normal((5, 4, 4)))
+    G = ed.ed_cpt_green(lat, Gc, kt, ed.ED_CPT_PERIODIZED)
+    far = ed.ed_cpt_green(dict(lat, pos=lat["pos"] + 2.0 ** 33), Gc, kt, ed.ED_CPT_PERIODIZED)
+    assert np.abs(far - G).max() <= 1e-13 * np.abs(G).max()
+
+
 @pytest.fixture(scope="module")
 def tridiag(tmp_path_factory):
     here = os.path.dirname(os.path.abspath(__file__))
