@@ -351,6 +351,7 @@ void launch_lanczos_step(const SectorView& sv, const HopParams& hp, int dtype, c
                          int nblk_cap, cudaStream_t s);
 int lanczos_blocks(const SectorView& sv);   // partial-sum slots per run of the fused step
 int two_pass_blocks(const SectorView& sv, int dtype);
+bool use_two_pass(const SectorView& sv, int dtype, const void* X, const void* O, int64_t vstride);  // whether products take the two-pass form
 
 // small.cu: many Lanczos levels of small sectors in one launch, a thread-block cluster per run.
 struct SmallStore {  // where the vectors v_{n0 + 1}, v_{n0 + 2}, ... are kept too

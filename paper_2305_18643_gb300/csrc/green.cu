@@ -303,9 +303,9 @@ static bool cf_part(ed_cluster& c, int spin, bool electron, int dtype, const Dev
     char* V[2] = {V0.p, V1.p};
     int cur = 0;
     int next_check = 32;
-    // small sectors: all levels up to the next check in one launch
+    // small sectors: all levels up to the next check in one launch, unless the two-pass form is asked for
     const double hops = (double)c.tables(nu_t).nnz / c.tables(nu_t).dim + (double)c.tables(nd_t).nnz / c.tables(nd_t).dim;
-    const int nb = small_cluster_size(sv, dtype, rc, hops);
+    const int nb = use_two_pass(sv, dtype, V[0], V[1], vstride) ? 0 : small_cluster_size(sv, dtype, rc, hops);
     for (int n = 0; n < M; ++n) {
       if (nb) {
         const int n1 = std::min(next_check, M);

@@ -636,7 +636,7 @@ static size_t down_rows_smem(const SectorView& sv, int dtype) {
 // The two-pass form applies when the vector has at least sv.two_pass_min_bytes (32 MiB unless the
 // cluster's ED_OPT_TWO_PASS_MIN_BYTES says otherwise: beyond that it no longer fits L2
 // comfortably) and the layout allows 16-byte vector access.
-static bool use_two_pass(const SectorView& sv, int dtype, const void* X, const void* O, int64_t vstride) {
+bool use_two_pass(const SectorView& sv, int dtype, const void* X, const void* O, int64_t vstride) {
   const int64_t es = dtype == ED_FP64 ? 8 : 4, NV = dtype == ED_FP64 ? 2 : 4;
   if (sv.d_up * sv.d_dn * es < sv.two_pass_min_bytes) return false;
   const int64_t need = (sv.d_dn + 32 * NV - 1) / (32 * NV) * (32 * NV);

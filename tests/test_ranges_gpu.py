@@ -85,6 +85,26 @@ def test_two_pass_option_selects_the_product(L, n_up, n_dn, dtype):
                                                 torch.cuda.current_stream().cuda_stream)) == launches
 
 
+# A forced two-pass form holds for continued fractions too (row pass, column pass and normalization per
+# level), and gives the G of the form that small sectors take by themselves, at sectors from a few states
+# up to and past the largest of the cluster kernel (1e-8, 2e-4 with FP32 vectors: the bounds of the parity tests).
+@pytest.mark.parametrize("L,n_up,n_dn", [(2, 1, 1), (8, 4, 4), (9, 4, 4), (12, 3, 2), (9, 4, 5), (17, 2, 2)])
+@pytest.mark.parametrize("precision,tol", [(ed.ED_FP64, 1e-8), (ed.ED_FP32, 2e-4)])
+def test_two_pass_option_selects_the_fractions(L, n_up, n_dn, precision, tol):
+    c = W.random_cluster(np.random.default_rng(L), L, 0, n_up, n_dn)
+    om = W.matsubara_grid(65)
+    G = []
+    for force in (False, True):
+        with ed.Cluster(c, seed=5, precision=precision) as cl:
+            if force:
+                ed.ed_set_option(cl.h, ed.ED_OPT_TWO_PASS_MIN_BYTES, 0)
+            cl.ground_state()
+            n = _launches(lambda: G.append(cl.green(om, 0.0, axis=ed.ED_AXIS_MATSUBARA)))
+            longest = ed.ed_green_stats(cl.h)[1]
+    assert n >= 3 * longest
+    assert np.abs(G[0] - G[1]).max() <= tol
+
+
 # Continued fractions of clusters whose energies are far beyond the frequencies: eight levels of the recurrences leave
 # the range of FP64 by the coefficients alone.  Within 1e-8 of the largest |G| of the exact Lehmann sum.
 @pytest.mark.parametrize("scale", [2.0 ** 40, 2.0 ** 130, 2.0 ** 200])
