@@ -354,13 +354,9 @@ int two_pass_blocks(const SectorView& sv, int dtype);
 bool use_two_pass(const SectorView& sv, int dtype, const void* X, const void* O, int64_t vstride);  // whether products take the two-pass form
 
 // small.cu: many Lanczos levels of small sectors in one launch, a thread-block cluster per run.
-struct SmallStore {  // where the vectors v_{n0 + 1}, v_{n0 + 2}, ... are kept too
-  void* p[16];
-  int count;
-};
 int small_cluster_size(const SectorView& sv, int dtype, int runs, double hops);
 void launch_small_levels(const SectorView& sv, const HopParams& hp, int dtype, void* V, void* VP, int64_t vstride, int runs,
-                         int n0, int n1, const LanczosScalars& ls, int nb, const SmallStore& store, cudaStream_t s);
+                         int n0, int n1, const LanczosScalars& ls, int nb, cudaStream_t s);
 
 // lanczos.cu
 // v_{n+1} = (W - a_n X) / b_{n+1} over W, or to dst; omega (contiguous) += coef[n + 1] v_{n+1}; its type is omega_dtype (< 0: the vectors' dtype).

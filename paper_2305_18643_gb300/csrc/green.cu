@@ -309,7 +309,7 @@ static bool cf_part(ed_cluster& c, int spin, bool electron, int dtype, const Dev
     for (int n = 0; n < M; ++n) {
       if (nb) {
         const int n1 = std::min(next_check, M);
-        launch_small_levels(sv, c.hp, dtype, V[0], V[1], vstride, rc, n, n1, ls, nb, SmallStore{}, s);
+        launch_small_levels(sv, c.hp, dtype, V[0], V[1], vstride, rc, n, n1, ls, nb, s);
         n = n1 - 1;
       } else {
         launch_lanczos_step(sv, c.hp, dtype, V[cur], V[cur ^ 1], vstride, rc, n, ls, nblk, s);

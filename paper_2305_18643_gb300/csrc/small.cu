@@ -50,8 +50,7 @@ __host__ __device__ inline size_t small_smem(int64_t dim, int slice, size_t es) 
 
 template <typename T>
 __global__ void __launch_bounds__(kSmallThreads) k_small_levels(SectorView sv, HopParams hp, T* __restrict__ V, T* __restrict__ VP,
-                                                                int64_t vstride, int slice, int n0, int n1, LanczosScalars ls,
-                                                                SmallStore store) {
+                                                                int64_t vstride, int slice, int n0, int n1, LanczosScalars ls) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), nb = (int)cluster.num_blocks();
   const int run = blockIdx.x / nb;
@@ -147,10 +146,6 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_levels(SectorView sv, H
       const T v = fma(-aT, x, W[i]) * ibT;
       P[i] = x;
       for (int r = 0; r < nb; ++r) cluster.map_shared_rank(X, r)[s0 + i] = v;
-      if (store.count) {
-        const int u = (int)(ud[i] >> 16), d = (int)(ud[i] & 0xffffu);
-        reinterpret_cast<T*>(store.p[n - n0])[(int64_t)u * sv.ld + d] = v;
-      }
     }
     cluster.sync();
   }
@@ -188,10 +183,9 @@ int small_cluster_size(const SectorView& sv, int dtype, int runs, double hops) {
 }
 
 // Levels [n0, n1) of `runs` runs (V = v_{n0}, VP = v_{n0 - 1}; on return the last two vectors), nb blocks
-// per run.  A run stops early as in launch_lanczos_step.  store: with count != 0, v_{n0 + 1 + k} goes to
-// store.p[k] too.
+// per run.  A run stops early as in launch_lanczos_step.
 void launch_small_levels(const SectorView& sv, const HopParams& hp, int dtype, void* V, void* VP, int64_t vstride, int runs,
-                         int n0, int n1, const LanczosScalars& ls, int nb, const SmallStore& store, cudaStream_t s) {
+                         int n0, int n1, const LanczosScalars& ls, int nb, cudaStream_t s) {
   const int64_t dim = sv.d_up * sv.d_dn;
   const int slice = (int)((dim + nb - 1) / nb);
   const size_t es = dtype == ED_FP64 ? 8 : 4;
@@ -209,10 +203,10 @@ void launch_small_levels(const SectorView& sv, const HopParams& hp, int dtype, v
   cfg.numAttrs = 1;
   if (dtype == ED_FP64) {
     allow_max_dynamic_smem(k_small_levels<double>);
-    ED_CUDA(cudaLaunchKernelEx(&cfg, k_small_levels<double>, sv, hp, (double*)V, (double*)VP, vstride, slice, n0, n1, ls, store));
+    ED_CUDA(cudaLaunchKernelEx(&cfg, k_small_levels<double>, sv, hp, (double*)V, (double*)VP, vstride, slice, n0, n1, ls));
   } else {
     allow_max_dynamic_smem(k_small_levels<float>);
-    ED_CUDA(cudaLaunchKernelEx(&cfg, k_small_levels<float>, sv, hp, (float*)V, (float*)VP, vstride, slice, n0, n1, ls, store));
+    ED_CUDA(cudaLaunchKernelEx(&cfg, k_small_levels<float>, sv, hp, (float*)V, (float*)VP, vstride, slice, n0, n1, ls));
   }
 }
 
