@@ -101,7 +101,10 @@ Footprint single_footprint(const ModelHost& m, const ed_cluster_desc& d, int nz,
       if (d.gf_method == ED_GF_CF) {
         const int64_t R = p + (int64_t)p * (p - 1) / 2;
         const int64_t M = std::max<int64_t>(64, std::min<int64_t>(cf_cap, 2 * reach + 16));
-        fx = (size_t)2 * R * nz * 16 + (size_t)R * (M * 16 + 64 * 16 + 64) + (size_t)nz * 16;
+        // per run: coefficients, and for every checked frequency the four numbers of its recurrences and its
+        // last value
+        const int zstride = std::max(1, nz / 1024), nzs = (nz + zstride - 1) / zstride;
+        fx = (size_t)2 * R * nz * 16 + (size_t)R * (M * 16 + (size_t)nzs * 5 * 16 + 64) + (size_t)nz * 16;
         mn = (size_t)2 * vstride * es;
         wn = (size_t)R * mn;
       } else {

@@ -86,3 +86,12 @@ def test_band_reserves_ring_unless_all_blocks_fit():
     cf_mid = ed.ed_request_bytes(c, n_freq=64, gf_budget=64 << 20)
     cf_hi = ed.ed_request_bytes(c, n_freq=64, gf_budget=0)
     assert cf_lo < cf_mid <= cf_hi
+
+
+def test_footprint_counts_the_fractions_check_state():
+    """Each continued fraction keeps five complex values per checked frequency (its recurrences and its last
+    value), beside its row of the table of fractions; every frequency is checked below 2,048."""
+    c = W.plain_2x4()
+    runs = 8 + 8 * 7 // 2
+    grown = ed.ed_request_bytes(c, n_freq=2047) - ed.ed_request_bytes(c, n_freq=1)
+    assert grown >= 2046 * runs * (5 * 16 + 2 * 16)
