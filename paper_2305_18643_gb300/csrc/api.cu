@@ -18,6 +18,7 @@ thread_local cudaMemPool_t g_alloc_pool = nullptr;
 namespace {
 std::mutex g_pools_mu;
 std::map<int, cudaMemPool_t> g_pools;
+std::map<int, int> g_pool_users;  // clusters with a stream of their own, by device
 }  // namespace
 
 cudaMemPool_t device_pool() {
@@ -39,6 +40,18 @@ cudaMemPool_t device_pool() {
     pool = nullptr;
   }
   return g_pools[dev] = pool;
+}
+
+void add_pool_user(int dev) {
+  std::lock_guard<std::mutex> lk(g_pools_mu);
+  ++g_pool_users[dev];
+}
+
+void drop_pool_user(int dev) {
+  std::lock_guard<std::mutex> lk(g_pools_mu);
+  if (--g_pool_users[dev] > 0) return;
+  auto it = g_pools.find(dev);
+  if (it != g_pools.end() && it->second) cudaMemPoolTrimTo(it->second, kPoolIdle);
 }
 
 void trim_device_pool() {
@@ -206,6 +219,7 @@ std::unique_ptr<ed_cluster> cluster_create_on(const ed_cluster_desc* desc, cudaS
   }
   c->tables(desc->n_up);
   c->tables(desc->n_dn);
+  if (c->owns_stream) add_pool_user(c->device);
   return c;
 }
 
@@ -265,8 +279,13 @@ void ed_cluster_destroy(ed_cluster* c) {
   try {
     cudaStreamSynchronize(c->stream);
     cudaStream_t s = c->owns_stream ? c->stream : nullptr;
+    const int dev = c->device;
     delete c;
-    if (s) cudaStreamDestroy(s);
+    if (s) {
+      cudaStreamSynchronize(s);  // the buffers are back in the pool
+      cudaStreamDestroy(s);
+      drop_pool_user(dev);
+    }
   } catch (...) {
   }
 }

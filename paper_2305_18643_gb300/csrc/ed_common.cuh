@@ -88,8 +88,10 @@ struct AllocStreamScope {
 
 // Memory of one solve (ground state, Green function) of a cluster with a stream of its own: DevBufs come
 // stream-ordered from a pool of the library, one per device, that keeps at most kPoolKeep bytes between
-// calls, returns the rest to the device when a stream is synchronized, and all that it holds unused when an
-// allocation of the library finds no memory.  cudaMalloc and cudaFree (which waits for the device) took 4 ms
+// calls, returns the rest to the device when a stream is synchronized, all that it holds unused when an
+// allocation of the library finds no memory, and all but kPoolIdle bytes when the device's last such cluster
+// is destroyed (with 64 MiB left the band solve of an 11-orbital chain takes 172.5 ms, with 512 MiB 166.4, with all
+// that the pool may keep 166.2).  cudaMalloc and cudaFree (which waits for the device) took 4 ms
 // of a 55 ms solve.  Only buffers used on the cluster's stream alone may come from it: the sector tables,
 // which ed_hpsi reads on the caller's stream, are allocated under PlainAllocScope.  Nested scopes (the
 // server's lanes) keep the outer one.  Buffers beyond kPoolMaxAlloc stay with cudaMalloc: the pool would
@@ -97,9 +99,12 @@ struct AllocStreamScope {
 // against 1.03 s).
 constexpr size_t kPoolMaxAlloc = size_t(256) << 20;
 constexpr size_t kPoolKeep = size_t(4) << 30;
+constexpr size_t kPoolIdle = size_t(512) << 20;
 extern thread_local cudaMemPool_t g_alloc_pool;
 cudaMemPool_t device_pool();  // the current device's pool; nullptr when the device has none
 void trim_device_pool();      // returns what that pool holds unused to the device
+void add_pool_user(int dev);  // counts the clusters that use the pool of device dev; with the last one
+void drop_pool_user(int dev);  // goes what it keeps beyond kPoolIdle
 struct PoolScope {
   cudaStream_t prev_s;
   cudaMemPool_t prev_p;
