@@ -30,8 +30,10 @@ constexpr int kThreads = 256;
 // hop and as little else in FP64 as possible (signs by integer operations, U sum n n by one
 // multiply-add on the popcount), all lanes of a warp on elements.
 //  - k_hpsi_flat: a thread per element of the flat index, for sectors of short rows (d_dn < 192),
-//    where rows dealt to blocks would leave most of their threads idle; with ROWS, rows over blocks, for
-//    rows too long for shared memory.
+//    where rows dealt to blocks would leave most of their threads idle; with ROWS, chunks of rows over
+//    blocks, for rows too long for shared memory (such sectors have few rows: 20 orbitals, (1, 10)
+//    particles, 20 rows of 184,756, took 1,560 us FP32 and 1,814 us FP64 with a block per row; 64 and 144 us
+//    in chunks).
 //  - k_hpsi_tile: TU rows at a time staged in shared memory as [d][TU], a thread per column: every
 //    down-spin entry serves TU rows, the up-spin entries of the rows are staged once per tile.
 // The fused forms compute w = H x - b_n x_prev over x_prev and reduce <x, w>, <w, w>, <x, x>; the last block
@@ -76,6 +78,8 @@ __device__ __forceinline__ void finish_step(double sxw, double sww, double sxx, 
   }
 }
 
+constexpr int64_t kRowChunk = 2 * kThreads;  // columns of a row that a block takes at a time
+
 template <typename T, bool FUSED, bool ROWS>
 __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams hp, const T* __restrict__ X0,
                                                         T* __restrict__ O0, int64_t vstride, int n, LanczosScalars ls) {
@@ -102,8 +106,12 @@ __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams
     O[o] = w;
   };
   if constexpr (ROWS) {
-    for (int64_t u = blockIdx.x; u < sv.d_up; u += gridDim.x)
-      for (int64_t d = threadIdx.x; d < sv.d_dn; d += blockDim.x) element(u, d);
+    const int64_t nchunk = (sv.d_dn + kRowChunk - 1) / kRowChunk, units = sv.d_up * nchunk;
+    for (int64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
+      const int64_t u = unit / nchunk, c0 = (unit - u * nchunk) * kRowChunk;
+      const int64_t c1 = c0 + kRowChunk < sv.d_dn ? c0 + kRowChunk : sv.d_dn;
+      for (int64_t d = c0 + threadIdx.x; d < c1; d += blockDim.x) element(u, d);
+    }
   } else {
     const uint32_t dim = (uint32_t)(sv.d_up * sv.d_dn), dd = (uint32_t)sv.d_dn;  // d_dn < 192 keeps it below 2^32
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += gridDim.x * blockDim.x) {

@@ -204,3 +204,11 @@ def test_last_cluster_returns_its_memory(method):
 
     free = solve(W.plain_2x4())
     assert solve(W.cdmft_2x2_bath()) >= free - (528 << 20)
+
+
+# Rows too long for shared memory, dealt to the blocks in chunks of columns, in the fused step of a whole solve.
+def test_long_rows_lanczos():
+    c = W.random_cluster(np.random.default_rng(18), 18, 0, 1, 8)
+    E = O.ground_state(O.sector_hamiltonian(_model(c), 1, 8))[0]
+    with ed.Cluster(c, seed=5) as cl:
+        assert abs(cl.ground_state()[1] - np.min(E)) <= 1e-10 * abs(np.min(E))
