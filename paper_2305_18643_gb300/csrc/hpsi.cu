@@ -122,7 +122,11 @@ __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams
   if (FUSED) finish_step(sxw, sww, sxx, run, n, ls);
 }
 
-constexpr int kTileThreads = 512;  // at most
+// Threads of a tiled block, at most.  FP32 products wait for their loads, so a tile that leaves no room for a second
+// block on its SM takes 1,024: 16 orbitals, (5, 8) particles, rows of 12,870, 1,308 us with 512, 762 us with 1,024
+// (992 us with rows dealt to blocks, 1,039 us in two blocks with tiles of half the rows).  FP64 is bound by its pipe.
+constexpr int kTileThreads = 512;
+constexpr int kTileThreadsAlone = 1024;
 constexpr int kFlatMaxRow = 192;   // shorter rows take the flat form
 
 // The staged tile: TU values of one column side by side.
@@ -138,7 +142,7 @@ struct alignas(16) UpHop {
 };
 
 template <typename T, int TU, bool FUSED>
-__global__ void __launch_bounds__(kTileThreads) k_hpsi_tile(SectorView sv, HopParams hp, const T* __restrict__ X0,
+__global__ void __launch_bounds__(sizeof(T) == 4 ? kTileThreadsAlone : kTileThreads) k_hpsi_tile(SectorView sv, HopParams hp, const T* __restrict__ X0,
                                                             T* __restrict__ O0, int64_t vstride, int nchunk, int chunk,
                                                             int zup, int n, LanczosScalars ls) {
   using Col = TileCol<T, TU>;
@@ -726,7 +730,7 @@ static TilePlan tile_plan(const SectorView& sv, int dtype) {
   p.nchunk = (int)std::min<int64_t>(want, (sv.d_dn + 255) / 256);
   p.chunk = (int)(((sv.d_dn + p.nchunk - 1) / p.nchunk + 31) / 32 * 32);
   p.nchunk = (int)((sv.d_dn + p.chunk - 1) / p.chunk);
-  p.threads = std::min(kTileThreads, p.chunk);
+  p.threads = std::min(dtype == ED_FP32 && p.smem > limit / 2 ? kTileThreadsAlone : kTileThreads, p.chunk);
   p.units = tiles * p.nchunk;
   return p;
 }
