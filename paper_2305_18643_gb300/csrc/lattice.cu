@@ -541,7 +541,7 @@ static void require_lat(bool ok, const char* msg) {
 // Distance (and gradient) of n_cand baths against A, all on the device; d and grad to the host.
 struct DistanceWork {
   int L, nb, nz;
-  DevBuf<double2> z, A, Gam, g;
+  DevBuf<double2> z, A, Gam;  // Gam: the hybridizations, then 1 / (z - eps) of every bath
   DevBuf<double> W, eps, theta, d, grad;
   void setup(int L_, int nb_, const double* zh, int nz_, const double* Wh, const double* Ah, cudaStream_t s) {
     L = L_;
@@ -557,7 +557,9 @@ struct DistanceWork {
   void eval(int nc, const double* eps_h, const double* theta_h, double* d_h, double* grad_h, cudaStream_t s) {
     if (eps.n < (size_t)std::max(nc * nb, 1)) eps.alloc(std::max(nc * nb, 1));
     if (theta.n < (size_t)std::max(nc * L * nb, 1)) theta.alloc(std::max(nc * L * nb, 1));
-    if (Gam.n < (size_t)nc * nz * L * L) Gam.alloc((size_t)nc * nz * L * L);
+    const size_t ngam = (size_t)nc * nz * L * L;
+    if (Gam.n < ngam + (size_t)nc * nz * nb) Gam.alloc(ngam + (size_t)nc * nz * nb);
+    double2* g = Gam.p + ngam;
     if (d.n < (size_t)nc) d.alloc(nc);
     const int np = nb + L * nb;
     if (grad_h && grad.n < (size_t)std::max(nc * np, 1)) grad.alloc(std::max(nc * np, 1));
@@ -565,15 +567,14 @@ struct DistanceWork {
       ED_CUDA(cudaMemcpyAsync(eps.p, eps_h, (size_t)nc * nb * sizeof(double), cudaMemcpyHostToDevice, s));
       ED_CUDA(cudaMemcpyAsync(theta.p, theta_h, (size_t)nc * L * nb * sizeof(double), cudaMemcpyHostToDevice, s));
     }
-    if (g.n < (size_t)std::max<int64_t>((int64_t)nc * nz * nb, 1)) g.alloc(std::max<int64_t>((int64_t)nc * nz * nb, 1));
     if (nb) {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_bath_g<<<lat_grid((int64_t)nc * nz * nb, 256), 256, 0, s>>>(eps.p, z.p, nb, nz, nc, g.p);
+      k_bath_g<<<lat_grid((int64_t)nc * nz * nb, 256), 256, 0, s>>>(eps.p, z.p, nb, nz, nc, g);
       ED_CHECK_LAUNCH();
     }
     {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_hybridization<<<lat_grid((int64_t)nc * nz * L * L, 256), 256, 0, s>>>(theta.p, g.p, L, nb, nz, nc, Gam.p);
+      k_hybridization<<<lat_grid((int64_t)nc * nz * L * L, 256), 256, 0, s>>>(theta.p, g, L, nb, nz, nc, Gam.p);
       ED_CHECK_LAUNCH();
     }
     {
@@ -584,7 +585,7 @@ struct DistanceWork {
     if (grad_h && np) {
       ProfScope ps_(K_LATTICE, s, 0.0);
       const int slices = std::max(1, std::min(32, 256 / np)), tile = 256 / slices;
-      k_distance_grad<<<dim3(nc, (np + tile - 1) / tile), 256, 0, s>>>(A.p, Gam.p, W.p, g.p, theta.p, L, nb, nz, slices,
+      k_distance_grad<<<dim3(nc, (np + tile - 1) / tile), 256, 0, s>>>(A.p, Gam.p, W.p, g, theta.p, L, nb, nz, slices,
                                                                        grad.p);
       ED_CHECK_LAUNCH();
     }
@@ -616,7 +617,8 @@ ed_status ed_hybridization(int n_sites, int n_bath, const double* eps, const dou
     cudaStream_t s = cudaStreamPerThread;
     const int L = n_sites;
     const size_t n = (size_t)nz * L * L;
-    DevBuf<double2> zd(nz), tmp;
+    DevBuf<double2> zd((size_t)nz * (1 + n_bath)), tmp;  // z, then 1 / (z - eps)
+    double2* g = zd.p + nz;
     DevBuf<double> ed_(std::max(n_bath, 1)), td((size_t)std::max(L * n_bath, 1));
     ED_CUDA(cudaMemcpyAsync(zd.p, z, nz * sizeof(double2), cudaMemcpyHostToDevice, s));
     if (n_bath) {
@@ -628,15 +630,14 @@ ed_status ed_hybridization(int n_sites, int n_bath, const double* eps, const dou
       tmp.alloc(n);
       out = tmp.p;
     }
-    DevBuf<double2> g(std::max<size_t>((size_t)nz * n_bath, 1));
     if (n_bath) {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_bath_g<<<lat_grid((int64_t)nz * n_bath, 256), 256, 0, s>>>(ed_.p, zd.p, n_bath, nz, 1, g.p);
+      k_bath_g<<<lat_grid((int64_t)nz * n_bath, 256), 256, 0, s>>>(ed_.p, zd.p, n_bath, nz, 1, g);
       ED_CHECK_LAUNCH();
     }
     {
       ProfScope ps_(K_LATTICE, s, 0.0);
-      k_hybridization<<<lat_grid((int64_t)n, 256), 256, 0, s>>>(td.p, g.p, L, n_bath, nz, 1, out);
+      k_hybridization<<<lat_grid((int64_t)n, 256), 256, 0, s>>>(td.p, g, L, n_bath, nz, 1, out);
       ED_CHECK_LAUNCH();
     }
     if (!out_is_device) ED_CUDA(cudaMemcpyAsync(Gamma_out, tmp.p, n * sizeof(double2), cudaMemcpyDeviceToHost, s));
