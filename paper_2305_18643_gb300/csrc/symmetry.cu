@@ -1063,8 +1063,11 @@ static void sym_cf_multi(ed_sym& T, int R, const SymMultiStart& st, double E0, d
   int* brk = reinterpret_cast<int*>(res.p + kSymMaxRuns);
   ED_CUDA(cudaMemsetAsync(tk.p, 0, sizeof(unsigned), s));
   ED_CUDA(cudaMemsetAsync(prev.p, 0, prev.n * sizeof(double2), s));
-  k_sym_multi_start<<<grid, threads, 0, s>>>(dim, R, st, U0.p, c, part.p, tk.p);
-  ED_CHECK_LAUNCH();
+  {
+    ProfScope ps_(K_VECTOR, s, (double)dim * 16.0 * R);
+    k_sym_multi_start<<<grid, threads, 0, s>>>(dim, R, st, U0.p, c, part.p, tk.p);
+    ED_CHECK_LAUNCH();
+  }
   double* u = U0.p;
   double* y = U1.p;
   int levels[kSymMaxRuns], quiet[kSymMaxRuns] = {};
@@ -1086,17 +1089,23 @@ static void sym_cf_multi(ed_sym& T, int R, const SymMultiStart& st, double E0, d
       k_sym_multi_spmv<<<grid, threads, 0, s>>>(T.rowptr.p, T.col.p, T.val.p, dim, R, u, y, n, c, part.p, tk.p);
       ED_CHECK_LAUNCH();
     }
-    k_sym_multi_axpy<<<grid, threads, 0, s>>>(dim, R, u, y, n, c, part.p, tk.p);
-    ED_CHECK_LAUNCH();
+    {
+      ProfScope ps_(K_VECTOR, s, (double)dim * 24.0 * R);
+      k_sym_multi_axpy<<<grid, threads, 0, s>>>(dim, R, u, y, n, c, part.p, tk.p);
+      ED_CHECK_LAUNCH();
+    }
     std::swap(u, y);
     if ((n + 1) % kSymCfCheck == 0 || n + 1 == maxn) {
       unsigned long long h[2 * kSymMaxRuns];
       int* hbrk = reinterpret_cast<int*>(h + kSymMaxRuns);
       ED_CUDA(cudaMemsetAsync(maxd, 0, kSymMaxRuns * sizeof(unsigned long long), s));
       ED_CUDA(cudaMemsetAsync(brk, 0x7f, kSymMaxRuns * sizeof(int), s));
-      k_sym_multi_check<<<dim3((nz + kSymEvalThreads - 1) / kSymEvalThreads, R), kSymEvalThreads, 0, s>>>(
-          c, checked, n + 1, E0, s_eh, zr.p, zi.p, nz, state.p, prev.p, bmin, maxd, brk);
-      ED_CHECK_LAUNCH();
+      {
+        ProfScope ps_(K_GF_EVAL, s, 0.0);
+        k_sym_multi_check<<<dim3((nz + kSymEvalThreads - 1) / kSymEvalThreads, R), kSymEvalThreads, 0, s>>>(
+            c, checked, n + 1, E0, s_eh, zr.p, zi.p, nz, state.p, prev.p, bmin, maxd, brk);
+        ED_CHECK_LAUNCH();
+      }
       ED_CUDA(cudaMemcpyAsync(h, res.p, sizeof(h), cudaMemcpyDeviceToHost, s));
       ED_CUDA(cudaStreamSynchronize(s));
       for (int r = 0; r < R; ++r) {
@@ -1118,6 +1127,7 @@ static void sym_cf_multi(ed_sym& T, int R, const SymMultiStart& st, double E0, d
   }
   for (int r = 0; r < R; ++r) {
     if (levels[r] == 0) continue;
+    ProfScope ps_(K_GF_EVAL, s, 0.0);
     k_sym_cf_eval<<<(nz + kSymEvalThreads - 1) / kSymEvalThreads, kSymEvalThreads, 0, s>>>(
         c.alpha + (size_t)r * stride, c.norm + (size_t)r * stride, levels[r], E0, b0[r] * b0[r], s_eh, zr.p, zi.p, nz, 1.0, out[r]);
     ED_CHECK_LAUNCH();

@@ -212,3 +212,21 @@ def test_long_rows_lanczos():
     E = O.ground_state(O.sector_hamiltonian(_model(c), 1, 8))[0]
     with ed.Cluster(c, seed=5) as cl:
         assert abs(cl.ground_state()[1] - np.min(E)) <= 1e-10 * abs(np.min(E))
+
+
+# The launches of a symmetrized Green function are counted and timed: beside every product of its runs there is
+# a vector update, and every run is evaluated.
+def test_symmetrized_fractions_are_counted():
+    c, mirrors = W.open_3x4_c2v()
+    kernels = {ed.ed_profile_kernel_name(k): k for k in range(11)}
+    with ed.Cluster(dict(c, n_up=2, n_dn=1), seed=5) as cl:
+        sym = ed.ed_sym_create(cl.h, mirrors, [1, 1])
+        try:
+            ed.ed_sym_ground_state(sym)
+            ed.ed_profile_enable(True)
+            ed.ed_sym_green(sym, W.matsubara_grid(16), 12, axis=ed.ED_AXIS_MATSUBARA)
+            n = {k: ed.ed_profile_read(kernels[k])[0] for k in ("hpsi", "vector", "gf_eval")}
+        finally:
+            ed.ed_profile_enable(False)
+            ed.ed_sym_destroy(sym)
+    assert n["vector"] >= n["hpsi"] > 0 and n["gf_eval"] > 0
