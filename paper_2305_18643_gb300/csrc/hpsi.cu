@@ -30,10 +30,11 @@ constexpr int kThreads = 256;
 // hop and as little else in FP64 as possible (signs by integer operations, U sum n n by one
 // multiply-add on the popcount), all lanes of a warp on elements.
 //  - k_hpsi_flat: a thread per element of the flat index, for sectors of short rows (d_dn < 192),
-//    where rows dealt to blocks would leave most of their threads idle; with ROWS, chunks of rows over
-//    blocks, for rows too long for shared memory (such sectors have few rows: 20 orbitals, (1, 10)
-//    particles, 20 rows of 184,756, took 1,560 us FP32 and 1,814 us FP64 with a block per row; 64 and 144 us
-//    in chunks).
+//    where rows dealt to blocks would leave most of their threads idle; with ROWS, rows over blocks, for
+//    rows too long for shared memory or (FP32) that fill an SM's by themselves.  Rows are cut into chunks of columns
+//    until every block has four: 20 rows of 184,756 (20 orbitals, (1, 10) particles) took 1,560 us FP32 and
+//    1,814 us FP64 whole, 62 and 144 us in chunks.  8,568 rows of 48,620 (18 orbitals, (5, 9)) stay whole, so that
+//    a row's operands stay in its SM's L1: 8.0 ms FP32, 9.3 ms in chunks of 512, 11.1 ms staged one row a tile.
 //  - k_hpsi_tile: TU rows at a time staged in shared memory as [d][TU], a thread per column: every
 //    down-spin entry serves TU rows, the up-spin entries of the rows are staged once per tile.
 // The fused forms compute w = H x - b_n x_prev over x_prev and reduce <x, w>, <w, w>, <x, x>; the last block
@@ -78,8 +79,6 @@ __device__ __forceinline__ void finish_step(double sxw, double sww, double sxx, 
   }
 }
 
-constexpr int64_t kRowChunk = 2 * kThreads;  // columns of a row that a block takes at a time
-
 template <typename T, bool FUSED, bool ROWS>
 __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams hp, const T* __restrict__ X0,
                                                         T* __restrict__ O0, int64_t vstride, int n, LanczosScalars ls) {
@@ -106,10 +105,12 @@ __global__ void __launch_bounds__(kThreads) k_hpsi_flat(SectorView sv, HopParams
     O[o] = w;
   };
   if constexpr (ROWS) {
-    const int64_t nchunk = (sv.d_dn + kRowChunk - 1) / kRowChunk, units = sv.d_up * nchunk;
+    const int64_t per = (4 * (int64_t)gridDim.x + sv.d_up - 1) / sv.d_up;  // chunks of a row
+    const int64_t chunk = ((sv.d_dn + per - 1) / per + 31) / 32 * 32;
+    const int64_t nchunk = (sv.d_dn + chunk - 1) / chunk, units = sv.d_up * nchunk;
     for (int64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
-      const int64_t u = unit / nchunk, c0 = (unit - u * nchunk) * kRowChunk;
-      const int64_t c1 = c0 + kRowChunk < sv.d_dn ? c0 + kRowChunk : sv.d_dn;
+      const int64_t u = unit / nchunk, c0 = (unit - u * nchunk) * chunk;
+      const int64_t c1 = c0 + chunk < sv.d_dn ? c0 + chunk : sv.d_dn;
       for (int64_t d = c0 + threadIdx.x; d < c1; d += blockDim.x) element(u, d);
     }
   } else {
@@ -702,7 +703,8 @@ int two_pass_blocks(const SectorView& sv, int dtype) {
 // Rows, chunks and shared memory of the tiled one-pass form for one vector (tu = 0: it does not
 // apply and the flat form runs).  Rows below 192 columns cannot fill their warps; four rows per
 // tile unless that leaves fewer than four tiles per SM (then the rows are split into chunks of columns,
-// each staging the tile again) or the tile exceeds shared memory.
+// each staging the tile again) or the tile exceeds shared memory.  One FP32 row by itself, without a second block beside
+// it, is not worth its staging.
 struct TilePlan {
   int tu = 0, nchunk = 1, chunk = 0, threads = 0, zup = 0;
   size_t smem = 0;
@@ -717,7 +719,7 @@ static TilePlan tile_plan(const SectorView& sv, int dtype) {
   const size_t limit = (size_t)smem_optin() - 8 * 1024;  // less the static shared memory
   for (int tu : {4, 2, 1}) {
     const size_t smem = ((size_t)sv.d_dn * tu * es + 15) / 16 * 16 + (size_t)tu * p.zup * 16;
-    if (smem > limit) continue;
+    if (smem > limit || (dtype == ED_FP32 && tu == 1 && smem > limit / 2)) continue;
     // small sectors: fewer rows per tile rather than idle SMs
     if (tu > 1 && (sv.d_up + tu - 1) / tu * ((sv.d_dn + 255) / 256) < 2 * 152) continue;
     p.tu = tu;

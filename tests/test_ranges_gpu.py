@@ -230,3 +230,11 @@ def test_symmetrized_fractions_are_counted():
             ed.ed_profile_enable(False)
             ed.ed_sym_destroy(sym)
     assert n["vector"] >= n["hpsi"] > 0 and n["gf_eval"] > 0
+
+
+# Single FP32 rows that would fill an SM's shared memory take the same form (rows of 43,758).
+def test_long_fp32_rows_lanczos():
+    c = W.random_cluster(np.random.default_rng(18), 18, 0, 1, 8)
+    with ed.Cluster(c, seed=5) as cl, ed.Cluster(c, seed=5, precision=ed.ED_FP32) as cl32:
+        E = cl.ground_state()[1]
+        assert abs(cl32.ground_state()[1] - E) <= 1e-10 * abs(E)
