@@ -85,7 +85,9 @@ const char* ed_last_error(void);
  * On success *out owns device memory until ed_cluster_destroy. */
 ed_status ed_cluster_create(const ed_cluster_desc* desc, ed_cluster** out);
 
-/* Frees every device buffer of the cluster.  NULL is ignored. */
+/* Frees every device buffer of the cluster.  NULL is ignored.  Solves take their buffers from a pool of the
+ * library, one per device, which keeps at most 4 GiB between calls while a cluster lives and at most
+ * 512 MiB once the device's last one is destroyed (clusters inside a server do not count). */
 void ed_cluster_destroy(ed_cluster* c);
 
 /* Lanczos ground state (Sec. 4.2): three-term recursion with FP64 reductions, lowest Ritz pair
@@ -121,7 +123,8 @@ ed_status ed_green(ed_cluster* c, const double* omega, int n_freq, double eta, i
  *                       two-pass kernels (a row pass for the down-spin hops and the diagonal, a
  *                       column pass for the up-spin hops) once a vector holds at least this many
  *                       bytes [33554432: beyond 32 MiB a vector no longer fits L2 comfortably];
- *                       0 selects them at every size.  Both forms compute the same product; the
+ *                       0 selects them at every size, in place of the kernel that runs many Lanczos
+ *                       levels of a small sector in one launch too.  Both forms compute the same product; the
  *                       option exists so that the two-pass kernels can be checked on sectors
  *                       small enough for a CPU reference.  Must be >= 0.
  *  ED_OPT_DAVIDSON_STATES
